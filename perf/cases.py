@@ -57,41 +57,41 @@ def listed():
     return [
         # one interactive user's step: four short requests over a small
         # vocabulary, issued call by call; launches and host time are all of it
-        _case("step tiny, calls", "step", 4, (64, 256), vocab=4096, logits="normal", how="calls",
+        _case("step tiny", "step", 4, (64, 256), vocab=4096, logits="normal", how="calls",
               rows="all"),
         # the everyday serving step: 64 student-driven requests, span 8, replayed
         # from a graph
-        _case("step 64 requests, graph", "step", 64, (1024, 8192), (8, 8), direction="S",
+        _case("step 64", "step", 64, (1024, 8192), (8, 8), direction="S",
               how="graph", rows="all"),
         # the full rollout step: 1024 requests, ragged spans, both drivers, only
         # the needed logits rows read
-        _case("step 1024 requests, graph", "step", 1024, (256, 32768, 4096), (1, 16), how="graph",
+        _case("step 1024", "step", 1024, (256, 32768, 4096), (1, 16), how="graph",
               rows="needed"),
         # a step whose logits come from a host-resident model: pinned inputs,
         # logits rows read in place over the host link
-        _case("step 256 requests, host-fed", "step", 256, (256, 32768, 4096), (1, 16), how="host",
+        _case("step 256 host-fed", "step", 256, (256, 32768, 4096), (1, 16), how="host",
               rows="needed"),
         # long reasoning traces: few requests, long contexts, 16-token spans
         # (128-row tiles) with the proposers' decode
-        _case("attention, long traces", "attn", 32, (8192, 32768), (16, 16), direction="S",
+        _case("attention long traces", "attn", 32, (8192, 32768), (16, 16), direction="S",
               decode_only=False),
         # student-verified ragged spans (2 to 32 rows per KV head) and GQA-8 decode
-        _case("attention, student verifies", "attn", 96, (256, 8192), (1, 16), direction="T",
+        _case("attention student verifies", "attn", 96, (256, 8192), (1, 16), direction="T",
               decode_only=False),
         # the proposal phase at a small batch: one decode token of 8 requests
-        _case("decode, 8 requests", "attn", 8, (500, 16000), (1, 1), direction="half",
+        _case("decode 8", "attn", 8, (500, 16000), (1, 1), direction="half",
               decode_only=True),
         # a high-batch step with entropy takeover, by-products and the next
         # span's first token
-        _case("score with rules, 512 requests", "score", 512, (2048, 4096), (4, 4), logits="zipf"),
+        _case("score with rules 512", "score", 512, (2048, 4096), (4, 4), logits="zipf"),
         # the training direction: top-K lists, loss, dense bf16 logit gradient
-        _case("loss and gradient, 77 requests", "train", 77, (1024, 8192), (1, 12), dense="bf16"),
+        _case("loss and gradient 77", "train", 77, (1024, 8192), (1, 12), dense="bf16"),
         # full-vocabulary KL of a monitoring pass over an odd number of positions
-        _case("full KL, 333 positions", "kl", 333, (1024, 8192), (1, 1)),
+        _case("full KL 333", "kl", 333, (1024, 8192), (1, 1)),
         # proposers' sampling: one row per request
-        _case("sample, 192 rows", "sample", 192, (1024, 8192), (1, 1), logits="normal", sigma=3.0),
+        _case("sample 192", "sample", 192, (1024, 8192), (1, 1), logits="normal", sigma=3.0),
         # the step's K/V rows into both caches, one launch
-        _case("append, 64 requests", "append", 64, (1024, 8192), (8, 8)),
+        _case("append 64", "append", 64, (1024, 8192), (8, 8)),
     ]
 
 
