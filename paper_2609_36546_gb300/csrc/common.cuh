@@ -31,6 +31,15 @@ IPD_DEVINL uint16_t f2bf16(float f) {
   return (uint16_t)(u >> 16);
 }
 
+// Maximum of 8 bf16 values (one 16-byte vector) as fp32, via packed bf16x2 max.
+IPD_DEVINL float bf16x8_max(const uint4 &r) {
+  uint32_t a, b, c;
+  asm("max.bf16x2 %0, %1, %2;" : "=r"(a) : "r"(r.x), "r"(r.y));
+  asm("max.bf16x2 %0, %1, %2;" : "=r"(b) : "r"(r.z), "r"(r.w));
+  asm("max.bf16x2 %0, %1, %2;" : "=r"(c) : "r"(a), "r"(b));
+  return fmaxf(bf16lo(c), bf16hi(c));
+}
+
 // ---------------------------------------------------------------------------
 // shared-memory addresses, mbarriers, bulk copies (PTX ISA 8.x, sm_90+)
 // ---------------------------------------------------------------------------

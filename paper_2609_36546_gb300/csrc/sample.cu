@@ -12,12 +12,21 @@
 // to fp32 on its own (no fused multiply-add).  This is the Gumbel-max trick in
 // base 2: l c - lg2(-lg2 u) = log2(e) (l / T - ln(-ln u)) - log2(ln 2).
 //
-// Kernels: the vocabulary of each sampled row is cut into chunks of 8192
-// entries, one CTA per (row, chunk).  A thread takes 8 consecutive entries at
-// a time (one 16-byte load, two Philox blocks) and keeps the largest
-// (score, -id) key; a CTA reduces its keys and stores one partial per chunk;
-// a second kernel reduces the chunks of each row (max is order-free, so the
-// result does not depend on the schedule).
+// Most entries are ruled out by an upper bound of their score instead of having
+// it evaluated: with x = 1 - u (exact), -log2 u >= x log2 e, so
+//   s_v <= l_v c - (log2 x + log2(log2 e)).
+// Eight entries at a time are held against the best score found so far (shared
+// by a CTA's warps) by their largest logit and largest random word, one
+// hardware log2 for the eight, where each score takes two eight-term
+// polynomials; the few vectors that reach it take the bound entry by entry,
+// and only the entries that still reach it get the defined score, so the draw
+// stays bit-exact.
+//
+// Kernels: the sampled rows' 8-entry vectors form one flat range cut into one
+// wave of equal pieces, one per CTA (a piece meets at most two rows).  A CTA
+// stores its largest (score, -id) key per row it meets; a second kernel
+// reduces each row's keys (max is order-free, so the result does not depend
+// on the schedule).
 #include <cuda_runtime.h>
 #include <stdint.h>
 
@@ -49,24 +58,57 @@ PhiloxKeys philox_keys(uint64_t seed) {
   return k;
 }
 
-// Philox4x32 with 10 rounds.
-__device__ __forceinline__ uint4 philox10(uint4 c, const PhiloxKeys &key) {
+// What the first two rounds of Philox leave constant over a row: the counter
+// is (v / 4, draw_lo, draw_hi, 0), so round 1's second product and round 2's
+// first do not depend on v.
+struct PhiloxRow {
+  uint32_t x2, z2, w2;  // round 2's xor terms of words 0 and 2, and its word 3
+};
+
+__device__ __forceinline__ void mul_wide(uint32_t a, uint32_t b, uint32_t &hi, uint32_t &lo) {
+  const uint64_t p = (uint64_t)a * b;
+  lo = (uint32_t)p;
+  hi = (uint32_t)(p >> 32);
+}
+
+__device__ __forceinline__ PhiloxRow philox_row(uint32_t draw_lo, uint32_t draw_hi,
+                                                const PhiloxKeys &key) {
+  uint32_t h1, l1, h2, l2;
+  mul_wide(kPhiloxM1, draw_hi, h1, l1);                      // round 1
+  mul_wide(kPhiloxM0, h1 ^ draw_lo ^ key.k0[0], h2, l2);     // round 2
+  return PhiloxRow{l1 ^ key.k0[1], h2 ^ key.k1[1], l2};
+}
+
+// Philox4x32 with 10 rounds of counter (g, draw_lo, draw_hi, 0).
+__device__ __forceinline__ uint4 philox10(uint32_t g, const PhiloxRow &r, const PhiloxKeys &key) {
+  uint32_t h0, l0, h1, l1;
+  mul_wide(kPhiloxM0, g, h0, l0);                  // round 1
+  mul_wide(kPhiloxM1, h0 ^ key.k1[0], h1, l1);     // round 2
+  uint4 c = make_uint4(h1 ^ r.x2, l1, l0 ^ r.z2, r.w2);
 #pragma unroll
-  for (int i = 0; i < 10; ++i) {
-    const uint32_t lo0 = kPhiloxM0 * c.x, hi0 = __umulhi(kPhiloxM0, c.x);
-    const uint32_t lo1 = kPhiloxM1 * c.z, hi1 = __umulhi(kPhiloxM1, c.z);
-    c = make_uint4(hi1 ^ c.y ^ key.k0[i], lo1, hi0 ^ c.w ^ key.k1[i], lo0);
+  for (int i = 2; i < 10; ++i) {
+    mul_wide(kPhiloxM0, c.x, h0, l0);
+    mul_wide(kPhiloxM1, c.z, h1, l1);
+    c = make_uint4(h1 ^ c.y ^ key.k0[i], l1, h0 ^ c.w ^ key.k1[i], l0);
   }
   return c;
 }
 
-// (score, -id) as one ordered 64-bit key; -0 is folded onto +0; 0 = no entry
-__device__ __forceinline__ unsigned long long score_key(float s, int v) {
-  if (v < 0) return 0ull;
+// a score's order code: monotone, -0 folded onto +0
+__device__ __forceinline__ uint32_t score_code(float s) {
   uint32_t b = __float_as_uint(s);
   if (b == 0x80000000u) b = 0u;
-  const uint32_t o = (b & 0x80000000u) ? ~b : (b | 0x80000000u);
-  return ((unsigned long long)o << 32) | (unsigned long long)(0xffffffffu - (uint32_t)v);
+  return (b & 0x80000000u) ? ~b : (b | 0x80000000u);
+}
+__device__ __forceinline__ float code_score(uint32_t o) {
+  return __uint_as_float((o & 0x80000000u) ? (o & 0x7fffffffu) : ~o);
+}
+
+// (score, -id) as one ordered 64-bit key; 0 = no entry
+__device__ __forceinline__ unsigned long long score_key(float s, int v) {
+  if (v < 0) return 0ull;
+  return ((unsigned long long)score_code(s) << 32) |
+         (unsigned long long)(0xffffffffu - (uint32_t)v);
 }
 
 __device__ __forceinline__ unsigned long long max_u64(unsigned long long a, unsigned long long b) {
@@ -77,6 +119,14 @@ IPD_DEVINL unsigned long long f2_mul(unsigned long long a, unsigned long long b)
   unsigned long long d;
   asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
   return d;
+}
+
+// log2 on the special-function unit (absolute error below 2^-22 on (0.5, 2),
+// relative 2^-22 elsewhere), for bounds only
+IPD_DEVINL float lg2_approx(float x) {
+  float y;
+  asm("lg2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+  return y;
 }
 
 // The fixed lg2 of the sampler, of two positive values at once: for x =
@@ -128,6 +178,107 @@ __device__ __forceinline__ void score_x2(uint32_t lbits2, uint32_t r0, uint32_t 
   f2_unpack(f2_sub(f2_mul(l, c2), g), s0, s1);
 }
 
+// Upper bounds of two scores, short of the constant log2(log2 e): fl(l c) -
+// lg2.approx(1 - u).  1 - u = (2 (2^23 - 1 - (bits >> 9)) + 1) 2^-24 is exact,
+// formed like u from the complemented bits.  The products are the score's own
+// (rounded once), so the bound meets the score through one monotone
+// subtraction.
+__device__ __forceinline__ void bound_x2(uint32_t lbits2, uint32_t r0, uint32_t r1,
+                                         unsigned long long c2, float &b0, float &b1) {
+  const unsigned long long x = f2_sub(
+      f2_pack(__uint_as_float((r0 >> 9) ^ 0x3fffffffu), __uint_as_float((r1 >> 9) ^ 0x3fffffffu)),
+      f2_pack(__uint_as_float(0x3f7fffffu), __uint_as_float(0x3f7fffffu)));
+  float x0, x1;
+  f2_unpack(x, x0, x1);
+  const unsigned long long g = f2_pack(lg2_approx(x0), lg2_approx(x1));
+  const unsigned long long l = f2_pack(bf16lo(lbits2), bf16hi(lbits2));
+  f2_unpack(f2_sub(f2_mul(l, c2), g), b0, b1);
+}
+
+// Bounds are clamped here (an infinite logit's), so that a number can be put
+// into their low bits.
+constexpr float kMaxBound = 3.0e38f, kFltMax = 3.402823466e38f;
+
+// The least bound_x2 value of an entry whose score can reach `best`: a score
+// is at most bound - log2(log2 e) (0.52877); 0.5 leaves 0.028 for the errors
+// of lg2.approx (below 1e-5 at |log2 x| <= 24) and of the score's own two
+// fixed logarithms (below 2e-5 together), and 2^-18 |best| covers the rounding
+// of the two subtractions and the three bits taken from a bound.
+__device__ __forceinline__ float bound_threshold(float best) {
+  return fminf(fmaf(fabsf(best), -3.814697265625e-6f, best + 0.5f), 2.9e38f);
+}
+
+__device__ __forceinline__ float max8(const float (&v)[8]) {
+  return fmax3(fmax3(v[0], v[1], v[2]), fmax3(v[3], v[4], v[5]), fmaxf(v[6], v[7]));
+}
+
+// The entries of row vectors [v_lo, v_hi): every thread's best score and its
+// id.  Equal scores keep the lower id (-0 == +0 too), and a thread whose
+// entries all score -inf keeps the first id it met (-1: none).  s_thr is the
+// largest threshold any warp of the CTA has published: a plain word, since any
+// value ever written to it is a valid threshold; finite, so that a row of -inf
+// ends the search at once.
+__device__ __forceinline__ void scan_row(const uint16_t *__restrict__ row, int v_lo, int v_hi,
+                                         uint32_t draw_lo, uint32_t draw_hi, const PhiloxKeys &key,
+                                         float cf, volatile float *s_thr, float &bs, int &bv) {
+  const int lane = threadIdx.x & 31;
+  const unsigned long long c2 = f2_pack(cf, cf);
+  const PhiloxRow pr = philox_row(draw_lo, draw_hi, key);
+  int vec = v_lo + (int)threadIdx.x;
+  bs = -INFINITY;
+  bv = vec < v_hi ? vec * 8 : -1;
+  uint4 nxt = make_uint4(0, 0, 0, 0);
+  if (vec < v_hi) nxt = __ldg(reinterpret_cast<const uint4 *>(row) + vec);
+  for (int first = vec - lane; first < v_hi; first += kSampleThreads, vec += kSampleThreads) {
+    const uint4 raw = nxt;
+    if (vec + kSampleThreads < v_hi)
+      nxt = __ldg(reinterpret_cast<const uint4 *>(row) + vec + kSampleThreads);
+    const uint4 ra = philox10(2u * (uint32_t)vec, pr, key);
+    const uint4 rb = philox10(2u * (uint32_t)vec + 1u, pr, key);
+    // the vector's bound: its largest logit with its largest random word.  With
+    // y = 2^32 - 1 - bits, y 2^-32 is at most 2 (1 - u), so the bound needs one
+    // more unit of slack than an entry's own; y = 0 gives +inf
+    const uint32_t r8 = max(max(max(ra.x, ra.y), max(ra.z, ra.w)),
+                            max(max(rb.x, rb.y), max(rb.z, rb.w)));
+    const float b8 = __fsub_rn(__fmul_rn(bf16x8_max(raw), cf), lg2_approx(__uint2float_rn(~r8)));
+    float thr = *s_thr;
+    if (!__any_sync(0xffffffffu, vec < v_hi && b8 >= thr - 33.f)) continue;
+    // the entries' own bounds, the entry's number in the low three bits
+    float ub[8];
+    bound_x2(raw.x, ra.x, ra.y, c2, ub[0], ub[1]);
+    bound_x2(raw.y, ra.z, ra.w, c2, ub[2], ub[3]);
+    bound_x2(raw.z, rb.x, rb.y, c2, ub[4], ub[5]);
+    bound_x2(raw.w, rb.z, rb.w, c2, ub[6], ub[7]);
+#pragma unroll
+    for (int j = 0; j < 8; ++j)
+      ub[j] = __uint_as_float((__float_as_uint(fminf(ub[j], kMaxBound)) & ~7u) | (uint32_t)j);
+    float top = vec < v_hi ? max8(ub) : -INFINITY;
+    // score each lane's largest bound that reaches the threshold, which follows
+    // the warp's best score; then the next, usually none
+    while (__any_sync(0xffffffffu, top >= thr)) {
+      const uint32_t e = __float_as_uint(top) & 7u;
+      const bool e0 = e & 1u, e1 = e & 2u, e2 = e & 4u;
+      const uint32_t rlo = e1 ? (e0 ? ra.w : ra.z) : (e0 ? ra.y : ra.x);
+      const uint32_t rhi = e1 ? (e0 ? rb.w : rb.z) : (e0 ? rb.y : rb.x);
+      const uint32_t lw = e2 ? (e1 ? raw.w : raw.z) : (e1 ? raw.y : raw.x);
+      const uint32_t rr = e2 ? rhi : rlo;
+      float s, unused;
+      score_x2(e0 ? lw >> 16 : lw, rr, rr, c2, s, unused);
+      const int v = vec * 8 + (int)e;
+      if (top >= thr && (s > bs || (s == bs && v < bv))) {
+        bs = s;
+        bv = v;
+      }
+      thr = fmaxf(thr, bound_threshold(code_score(__reduce_max_sync(0xffffffffu, score_code(bs)))));
+      float rest[8];
+#pragma unroll
+      for (int j = 0; j < 8; ++j) rest[j] = ub[j] < top ? ub[j] : -INFINITY;
+      top = max8(rest);
+    }
+    if (lane == 0 && thr > *s_thr) *s_thr = thr;
+  }
+}
+
 // One draw per row of a list of rows.  mode 0: row r is row r of `rows0`
 // with draw number draw_id[r].  mode 1 (after a verdict): request r draws the
 // first token of its next span from the next driver's row n_emit[r] of its
@@ -135,11 +286,17 @@ __device__ __forceinline__ void score_x2(uint32_t lbits2, uint32_t r0, uint32_t 
 // prefix_len[r] + n_emit[r]; a request that ended or emitted every span token
 // draws nothing.
 //
+// Bound: the integer pipes.  Philox's 36 wide multiplies a vector keep the
+// heavy half of the FMA pipe half busy and the whole takes 24 warp
+// instructions an entry (44 when every entry was scored); the rows are read at
+// 1.5 TB/s.  192 rows of 151,936: 57.3 -> 41.3 us a call; four CTAs an SM
+// rather than five, which spilled (44.0 against 47.3 us in an earlier form).
+//
 // Work split: the rows' 8-entry vectors form one flat range that is cut into
 // gridDim.x equal pieces, one per CTA (grid >= rows, so a piece meets at most
 // two rows).  Each CTA stores its best key for the first and the second row
 // it meets (0 where it meets none).
-__global__ void __launch_bounds__(kSampleThreads, 5) sample_partial_kernel(
+__global__ void __launch_bounds__(kSampleThreads, 4) sample_partial_kernel(
     int mode, const uint16_t *__restrict__ rows0, const uint16_t *__restrict__ rows1, int vocab,
     int n_rows, const PhiloxKeys key, const uint64_t *__restrict__ draw_id,
     float inv_temperature, const int32_t *__restrict__ cu_span,
@@ -149,11 +306,11 @@ __global__ void __launch_bounds__(kSampleThreads, 5) sample_partial_kernel(
   __shared__ unsigned long long s_best[2][kSampleThreads / 32];
   __shared__ const uint16_t *s_row[2];
   __shared__ uint32_t s_draw[2][2];
+  __shared__ float s_thr[2];
   const long long nv = vocab >> 3;  // vectors per row
   const long long total = nv * n_rows;
   const long long lo = total * blockIdx.x / gridDim.x, hi = total * (blockIdx.x + 1) / gridDim.x;
   const int row_lo = (int)(lo / nv);
-  const long long boundary = (long long)(row_lo + 1) * nv;
   if (threadIdx.x < 2) {
     const int r = row_lo + (int)threadIdx.x;
     const uint16_t *row = nullptr;
@@ -173,55 +330,21 @@ __global__ void __launch_bounds__(kSampleThreads, 5) sample_partial_kernel(
     s_row[threadIdx.x] = row;
     s_draw[threadIdx.x][0] = (uint32_t)draw;
     s_draw[threadIdx.x][1] = (uint32_t)(draw >> 32);
+    s_thr[threadIdx.x] = -kFltMax;  // every finite bound reaches it, -inf never does
   }
   __syncthreads();
   const float cf = __fmul_rn(__uint_as_float(kLog2eBits), inv_temperature);
-  const unsigned long long c2 = f2_pack(cf, cf);
-  // per thread and row: the best score and its id; entries come in increasing
-  // id, so a strict comparison keeps the lower id of equal scores (-0 == +0
-  // too), and a row whose entries all score -inf keeps its first id
-  float bs0 = -INFINITY, bs1 = -INFINITY;
-  int bv0 = -1, bv1 = -1;
-  for (long long vec = lo + threadIdx.x; vec < hi; vec += kSampleThreads) {
-    const int k = vec >= boundary ? 1 : 0;
-    const uint16_t *row = s_row[k];
-    if (row == nullptr) continue;
-    const int v0 = (int)(vec - (long long)(row_lo + k) * nv) * 8;
-    float cbs = k ? bs1 : bs0;
-    int cbv = k ? bv1 : bv0;
-    if (cbv < 0) cbv = v0;
-    const uint4 raw = __ldg(reinterpret_cast<const uint4 *>(row + v0));
-    const uint32_t g = (uint32_t)v0 >> 2;
-    const uint4 ra = philox10(make_uint4(g, s_draw[k][0], s_draw[k][1], 0u), key);
-    const uint4 rb = philox10(make_uint4(g + 1u, s_draw[k][0], s_draw[k][1], 0u), key);
-    float sc[8];
-    score_x2(raw.x, ra.x, ra.y, c2, sc[0], sc[1]);
-    score_x2(raw.y, ra.z, ra.w, c2, sc[2], sc[3]);
-    score_x2(raw.z, rb.x, rb.y, c2, sc[4], sc[5]);
-    score_x2(raw.w, rb.z, rb.w, c2, sc[6], sc[7]);
-    // the vector's best; a new record (rare after the first vectors) looks up
-    // its first entry
-    const float m8 = fmaxf(fmaxf(fmaxf(sc[0], sc[1]), fmaxf(sc[2], sc[3])),
-                           fmaxf(fmaxf(sc[4], sc[5]), fmaxf(sc[6], sc[7])));
-    if (m8 > cbs) {
-      int e = 0;
-#pragma unroll
-      for (int j = 7; j >= 0; --j)
-        if (sc[j] == m8) e = j;
-      cbs = m8;
-      cbv = v0 + e;
-    }
-    if (k) {
-      bs1 = cbs;
-      bv1 = cbv;
-    } else {
-      bs0 = cbs;
-      bv0 = cbv;
-    }
-  }
-#pragma unroll
+#pragma unroll 1
   for (int k = 0; k < 2; ++k) {
-    unsigned long long b = k ? score_key(bs1, bv1) : score_key(bs0, bv0);
+    // this CTA's vectors of row row_lo + k
+    const long long base = (long long)(row_lo + k) * nv;
+    const int v_lo = (int)(lo > base ? lo - base : 0);
+    const int v_hi = (int)(hi - base < nv ? (hi > base ? hi - base : 0) : nv);
+    float bs = -INFINITY;
+    int bv = -1;
+    if (s_row[k] != nullptr)
+      scan_row(s_row[k], v_lo, v_hi, s_draw[k][0], s_draw[k][1], key, cf, &s_thr[k], bs, bv);
+    unsigned long long b = score_key(bs, bv);
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) b = max_u64(b, __shfl_xor_sync(0xffffffffu, b, o));
     if ((threadIdx.x & 31) == 0) s_best[k][threadIdx.x >> 5] = b;

@@ -67,15 +67,6 @@ __device__ __forceinline__ uint32_t elem_bits(const uint4 &r, int e) {
   return (e & 1) ? (w >> 16) : (w & 0xffffu);
 }
 
-// Maximum of 8 bf16 values (one 16-byte vector) as fp32, via packed bf16x2 max.
-__device__ __forceinline__ float bf16x8_max(const uint4 &r) {
-  uint32_t a, b, c;
-  asm("max.bf16x2 %0, %1, %2;" : "=r"(a) : "r"(r.x), "r"(r.y));
-  asm("max.bf16x2 %0, %1, %2;" : "=r"(b) : "r"(r.z), "r"(r.w));
-  asm("max.bf16x2 %0, %1, %2;" : "=r"(c) : "r"(a), "r"(b));
-  return fmaxf(bf16lo(c), bf16hi(c));
-}
-
 __device__ __forceinline__ unsigned long long shfl_u64(unsigned long long v, int src) {
   return __shfl_sync(0xffffffffu, v, src);
 }

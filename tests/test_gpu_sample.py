@@ -64,6 +64,35 @@ def test_sample_degenerate_rows(lib):
     assert got[1] == 1234 and got[2] == 0 and got[3] == 4095
 
 
+@pytest.mark.parametrize("V,n,inv_t", [(4096, 12, 1.0), (151936, 3, 1.0), (1040, 9, 1e-3),
+                                       (2056, 9, 300.0)])
+def test_sample_bounds_keep_the_draw(lib, V, n, inv_t):
+    """Rows on which the score bound that rules entries out is least useful or
+    closest to the scores: every score nearly equal, huge and tiny logits (the
+    bound's rounding grows with them), infinities, a single finite entry at the
+    end, ties of equal logits."""
+    g = torch.Generator().manual_seed(V)
+    rows = torch.zeros(n, V, dtype=torch.float32)
+    rows[1] = 1e30 * (1 + torch.rand(V, generator=g))   # spacing far above a draw's spread
+    rows[2] = -1e30 * (1 + torch.rand(V, generator=g))
+    if n > 3:
+        rows[3] = 40.0 * torch.randn(V, generator=g)
+        rows[4] = 1e-30 * torch.randn(V, generator=g)
+        rows[5] = float("-inf")
+        rows[5, V - 1] = -5.0
+        rows[6, V // 2] = rows[6, V // 2 + 9] = rows[6, V - 8] = float("inf")
+        rows[7] = torch.randn(V, generator=g)
+        rows[7, ::3] = float("-inf")
+        rows[8] = torch.where(torch.arange(V) % 511 == 7, 3.0e38, -3.0e38)
+    rows = rows.to(torch.bfloat16)
+    draws = np.arange(n, dtype=np.uint64) + np.uint64(77)
+    got = _gpu_sample(lib, rows, 11, draws, inv_t)
+    bits = u16(rows)
+    with np.errstate(over="ignore", invalid="ignore"):
+        assert got.tolist() == [O.sample_token(bits[i], 11, int(draws[i]), inv_t)
+                                for i in range(n)]
+
+
 def test_sample_many_draws_of_one_row(lib):
     """Different draw numbers of one row give independent draws; the ids follow
     the oracle draw by draw."""
