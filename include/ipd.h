@@ -210,6 +210,9 @@ int ipd_score_span(const uint16_t *logits_student, const uint16_t *logits_teache
  * rest are read as by ipd_score_span, position 0 of every request first.
  * A call whose rows all fit one wave of row CTAs reads every row (no
  * transition is known before every row has started).
+ * Logits in page-locked host memory (both models', see ipd_device_readable) are
+ * read over the host link by a few SMs, so that other kernels (the step's
+ * attention, launched after this call on another stream) run beside the pass.
  *
  * Arguments as for ipd_score_span, plus
  *  max_span       an upper bound (1 .. 65535) on every request's span length;

@@ -139,53 +139,59 @@ __device__ __forceinline__ unsigned long long warp_top32_u64(unsigned long long 
 struct NeededRows {
   const int32_t *tokens, *cu_span;
   const uint8_t *driver;
-  int *trans;  // [R] lowest transition position seen so far (starts high)
+  int *trans;  // [R] lowest transition position seen so far (starts at kTransStart)
   int total_tokens;
 };
+constexpr unsigned kTransStart = 0x7f7f7f7fu;  // above any position; set bytewise
 
+// Shared memory of one row's 128 threads.
+struct RowSmem {
+  uint16_t gmax[kMaxGroups][kRowThreads];  // group maxima (order codes, 0: none)
+  float sorted[kRowWarps][32];
+  float tau;
+  unsigned long long lists[kRowWarps][32];
+  unsigned long long buf[kRowWarps][kBuf];
+  int cand[kRowWarps][32 * kMaxGroupVecs];  // a round's candidate vectors
+  float m[kRowWarps], s[kRowWarps], u[kRowWarps];
+};
+static_assert(IPD_MAX_K == 32, "one key per lane");
+
+// Where a row of the needed-rows pass stands: request r's span position pos,
+// the row's model, the request's driver and its verifier's model.
+struct NeededPos {
+  int r, pos, t, model, drv, ver;
+};
+
+// Index i (< R the verifier's row, else the proposer's) of span position pos:
+// false if request i mod R has no such position (or offsets the epilogue
+// reports as broken).
+__device__ __forceinline__ bool needed_pos(const NeededRows &nr, int R, int i, int pos,
+                                           NeededPos *np) {
+  const bool is_ver = i < R;
+  const int r = is_ver ? i : i - R;
+  const int t0 = nr.cu_span[r], k = nr.cu_span[r + 1] - t0;
+  if (pos >= k || t0 < 0 || t0 + k > nr.total_tokens) return false;
+  const int drv = nr.driver[r] ? 1 : 0;
+  const int ver = drv ? 0 : 1;  // the verifier's row: the teacher's when the student drives
+  *np = NeededPos{r, pos, t0 + pos, is_ver ? ver : 1 - ver, drv, ver};
+  return true;
+}
+// whether the row is needed as far as the request's transition bound now tells
+__device__ __forceinline__ bool needed_now(const NeededRows &nr, const NeededPos &np) {
+  const int tr = *reinterpret_cast<volatile const int *>(nr.trans + np.r);
+  return np.model == np.ver || np.drv ? np.pos <= tr : np.pos < tr;
+}
+
+// One part (of `parts`) of one row, by 128 threads that meet at `sync`.
 template <bool kEntropy,  // also accumulate sum exp(l - m) l (entropies / entropy rules)
-          bool kNeeded>   // the needed-rows pass (one part per row)
-__global__ void __launch_bounds__(kRowThreads, kRowCtasPerSm) score_rows_kernel(
-    const uint16_t *__restrict__ ls, const uint16_t *__restrict__ lt, int vocab, int K, int parts,
-    RowOut *__restrict__ out, const NeededRows nr) {
+          bool kNeeded,   // the needed-rows pass (one part per row)
+          typename Sync>
+__device__ __forceinline__ void score_row(RowSmem &sm, const uint16_t *__restrict__ row, int vocab,
+                                          int K, int part, int parts, int tid,
+                                          RowOut *__restrict__ out, const NeededRows &nr,
+                                          const NeededPos &np, Sync sync) {
   constexpr int U = 4;  // vectors per thread and iteration
-  __shared__ uint16_t s_gmax[kMaxGroups][kRowThreads];  // group maxima (order codes, 0: none)
-  __shared__ float s_sorted[kRowWarps][32];
-  __shared__ float s_tau;
-  static_assert(IPD_MAX_K == 32, "one key per lane");
-  __shared__ unsigned long long s_lists[kRowWarps][32];
-  __shared__ unsigned long long s_buf[kRowWarps][kBuf];
-  __shared__ int s_cand[kRowWarps][32 * kMaxGroupVecs];  // a round's candidate vectors
-  __shared__ float s_m[kRowWarps], s_s[kRowWarps], s_u[kRowWarps];
-
-  int row_id = blockIdx.x / parts, part = blockIdx.x % parts, oi = blockIdx.x;
-  int r = 0, pos = 0, drv = 0, ver = 0;
-  if (kNeeded) {
-    // blocks 0 .. R-1 of a position take the verifiers' rows, R .. 2R-1 the
-    // proposers', so a proposer's row starts after its verifier's when the
-    // position spans more than one wave
-    const int R = gridDim.x >> 1;
-    const bool is_ver = (int)blockIdx.x < R;
-    r = is_ver ? blockIdx.x : blockIdx.x - R;
-    pos = blockIdx.y;
-    const int t0 = nr.cu_span[r], k = nr.cu_span[r + 1] - t0;
-    // no such position (or offsets the epilogue reports as broken)
-    if (pos >= k || t0 < 0 || t0 + k > nr.total_tokens) return;
-    drv = nr.driver[r] ? 1 : 0;
-    ver = drv ? 0 : 1;  // the verifier's row: the teacher's when the student drives
-    row_id = 2 * (t0 + pos) + (is_ver ? ver : 1 - ver);
-    part = 0;
-    oi = row_id;
-    const int tr = *reinterpret_cast<volatile const int *>(nr.trans + r);
-    const bool need = (row_id & 1) == ver ? pos <= tr : (drv ? pos <= tr : pos < tr);
-    if (!need) {
-      if (threadIdx.x == 0) out[oi].skipped = 1;
-      return;
-    }
-  }
-  const int t = row_id >> 1, model = row_id & 1;
-  const uint16_t *row = (model ? lt : ls) + (size_t)t * vocab;
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, tid = threadIdx.x;
+  const int lane = tid & 31, warp = tid >> 5;
   const int nvec = vocab >> 3;
   const int per = (nvec + parts - 1) / parts;
   const int v_lo = min(nvec, part * per), v_hi = min(nvec, v_lo + per);
@@ -193,7 +199,7 @@ __global__ void __launch_bounds__(kRowThreads, kRowCtasPerSm) score_rows_kernel(
   // iterations per group: two, or more so that a thread has at most kMaxGroups
   const int ipg = max(2, (n_iter + kMaxGroups - 1) / kMaxGroups);
   const int n_groups = (n_iter + ipg - 1) / ipg;
-  unsigned long long *buf = s_buf[warp];
+  unsigned long long *buf = sm.buf[warp];
 
   float m = -INFINITY;
   unsigned long long s2 = 0ull;  // running sum of exp(l - m), as a packed pair
@@ -232,7 +238,7 @@ __global__ void __launch_bounds__(kRowThreads, kRowCtasPerSm) score_rows_kernel(
       // vectors past the part read as -inf; a group with none of the part's
       // vectors keeps code 0 (a real logit, -inf included, has a code >= 1)
       const bool real = v_lo + (it / ipg) * ipg * kRowThreads * U + tid < v_hi;
-      s_gmax[it / ipg][tid] = real ? (uint16_t)ord16(__float_as_uint(gmax) >> 16) : (uint16_t)0;
+      sm.gmax[it / ipg][tid] = real ? (uint16_t)ord16(__float_as_uint(gmax) >> 16) : (uint16_t)0;
       gmax = -INFINITY;
     }
     if (bmax > m) {
@@ -269,18 +275,18 @@ __global__ void __launch_bounds__(kRowThreads, kRowCtasPerSm) score_rows_kernel(
   // with fewer than K counted maxima every group of the part qualifies.
   {
     const bool real = v_lo + tid < v_hi;
-    s_sorted[warp][lane] = warp_sort_desc_f(real ? m : -INFINITY, lane);
-    __syncthreads();
+    sm.sorted[warp][lane] = warp_sort_desc_f(real ? m : -INFINITY, lane);
+    sync();
     if (warp == 0) {  // the top 32 of the four sorted lists, then its K-th entry
       static_assert(kRowWarps == 4, "two rounds of pairwise merges");
-      const float a = warp_top32_f(s_sorted[0][lane], s_sorted[1][lane], lane);
-      const float b = warp_top32_f(s_sorted[2][lane], s_sorted[3][lane], lane);
+      const float a = warp_top32_f(sm.sorted[0][lane], sm.sorted[1][lane], lane);
+      const float b = warp_top32_f(sm.sorted[2][lane], sm.sorted[3][lane], lane);
       const float c = warp_top32_f(a, b, lane);
-      if (lane == K - 1) s_tau = c;  // -inf when fewer than K logits were read
+      if (lane == K - 1) sm.tau = c;  // -inf when fewer than K logits were read
     }
-    __syncthreads();
+    sync();
   }
-  const float tau = s_tau;
+  const float tau = sm.tau;
   const uint32_t g_code = tau == -INFINITY ? 1u : ord16(__float_as_uint(tau) >> 16);
 
   // ---- examine the groups that reach tau ----
@@ -313,7 +319,7 @@ __global__ void __launch_bounds__(kRowThreads, kRowCtasPerSm) score_rows_kernel(
   // single round.
   int j_next = 0, q_next = 0;  // this lane's next group, and next vector in it
   while (true) {
-    while (j_next < n_groups && s_gmax[j_next][tid] < g_code) ++j_next;
+    while (j_next < n_groups && sm.gmax[j_next][tid] < g_code) ++j_next;
     const bool have = j_next < n_groups;
     if (!__any_sync(0xffffffffu, have)) break;
     const int it0 = j_next * ipg;
@@ -327,7 +333,7 @@ __global__ void __launch_bounds__(kRowThreads, kRowCtasPerSm) score_rows_kernel(
     }
     const int total = __shfl_sync(0xffffffffu, off, 31);
     off -= n_lane;
-    int *cand = s_cand[warp];
+    int *cand = sm.cand[warp];
     for (int q = 0; q < n_lane; ++q) {
       const int qq = q_next + q;
       cand[off + q] = v_lo + (it0 + qq / U) * kRowThreads * U + (qq % U) * kRowThreads + tid;
@@ -380,36 +386,128 @@ __global__ void __launch_bounds__(kRowThreads, kRowCtasPerSm) score_rows_kernel(
   const float wf = (m == -INFINITY || wm == -INFINITY) ? 0.f : exp2f((m - wm) * kLog2e);
   float ws = warp_sum(s * wf);
   float wu = warp_sum(u * wf);
-  s_lists[warp][lane] = lane < nb ? buf[lane] : 0ull;
+  sm.lists[warp][lane] = lane < nb ? buf[lane] : 0ull;
   if (lane == 0) {
-    s_m[warp] = wm;
-    s_s[warp] = ws;
-    s_u[warp] = wu;
+    sm.m[warp] = wm;
+    sm.s[warp] = ws;
+    sm.u[warp] = wu;
   }
-  __syncthreads();
+  sync();
   if (warp == 0) {
-    float bm = lane < kRowWarps ? s_m[lane] : -INFINITY;
+    float bm = lane < kRowWarps ? sm.m[lane] : -INFINITY;
     const float gm = warp_max(bm);
     const float bf = (lane < kRowWarps && bm != -INFINITY) ? exp2f((bm - gm) * kLog2e) : 0.f;
-    const float bs = warp_sum(lane < kRowWarps ? s_s[lane] * bf : 0.f);
-    const float bu = warp_sum(lane < kRowWarps ? s_u[lane] * bf : 0.f);
+    const float bs = warp_sum(lane < kRowWarps ? sm.s[lane] * bf : 0.f);
+    const float bu = warp_sum(lane < kRowWarps ? sm.u[lane] * bf : 0.f);
     if (lane == 0) {
-      out[oi].m = gm;
-      out[oi].s = bs;
-      out[oi].u = bu;
-      if (kNeeded) out[oi].skipped = 0;
+      out->m = gm;
+      out->s = bs;
+      out->u = bu;
+      if (kNeeded) out->skipped = 0;
     }
     // the warps' lists (each sorted, 0 past its end) merged to the part's top K
-    const unsigned long long a = warp_top32_u64(s_lists[0][lane], s_lists[1][lane], lane);
-    const unsigned long long b = warp_top32_u64(s_lists[2][lane], s_lists[3][lane], lane);
+    const unsigned long long a = warp_top32_u64(sm.lists[0][lane], sm.lists[1][lane], lane);
+    const unsigned long long b = warp_top32_u64(sm.lists[2][lane], sm.lists[3][lane], lane);
     const unsigned long long c = warp_top32_u64(a, b, lane);
-    out[oi].keys[lane] = lane < K ? c : 0ull;
-    if (kNeeded && model == ver) {
+    out->keys[lane] = lane < K ? c : 0ull;
+    if (kNeeded && np.model == np.ver) {
       // coverage of the proposed token by this verifier row's Top_K
-      const int x = nr.tokens[t];
+      const int x = nr.tokens[np.t];
       const bool hit = lane < K && x >= 0 && x < vocab && key_idx(c) == (uint32_t)x;
       const bool cov = __ballot_sync(0xffffffffu, hit) != 0;
-      if (lane == 0 && (drv ? cov : !cov)) atomicMin(nr.trans + r, pos);
+      if (lane == 0 && (np.drv ? cov : !cov)) atomicMin(nr.trans + np.r, np.pos);
+    }
+  }
+}
+
+// CTA i takes part i % parts of row i / parts; in the needed-rows pass block
+// (i, pos) takes the verifier's (i < R) or the proposer's row of request
+// i mod R's position pos.
+template <bool kEntropy, bool kNeeded>
+__global__ void __launch_bounds__(kRowThreads, kRowCtasPerSm) score_rows_kernel(
+    const uint16_t *__restrict__ ls, const uint16_t *__restrict__ lt, int vocab, int K, int parts,
+    RowOut *__restrict__ out, const NeededRows nr) {
+  __shared__ RowSmem sm;
+  int row_id = blockIdx.x / parts, part = blockIdx.x % parts, oi = blockIdx.x;
+  NeededPos np{};
+  if (kNeeded) {
+    // blocks 0 .. R-1 of a position take the verifiers' rows, R .. 2R-1 the
+    // proposers', so a proposer's row starts after its verifier's when the
+    // position spans more than one wave
+    if (!needed_pos(nr, gridDim.x >> 1, blockIdx.x, blockIdx.y, &np)) return;
+    row_id = 2 * np.t + np.model;
+    part = 0;
+    oi = row_id;
+    if (!needed_now(nr, np)) {
+      if (threadIdx.x == 0) out[oi].skipped = 1;
+      return;
+    }
+  }
+  const int t = row_id >> 1, model = row_id & 1;
+  score_row<kEntropy, kNeeded>(sm, (model ? lt : ls) + (size_t)t * vocab, vocab, K, part, parts,
+                               threadIdx.x, out + oi, nr, np, [] { __syncthreads(); });
+}
+
+// The needed-rows pass over logits in host memory, read over the host link.
+// Bound: the link (about 206 GB/s against 6.8 TB/s of HBM), which a few SMs
+// saturate: 64 rows in flight, 16 KB of loads each, cover its latency with a
+// wide margin.  So this pass takes kLinkCtas SMs for its whole length and
+// leaves the others to the attention it runs beside, and because few rows are
+// in flight at once, most of the rows past a transition are never read.  A CTA
+// is eight groups of 128 threads, each taking rows one by one from a shared
+// counter in the order of the grid above (four indices a claim, their need
+// looked up side by side, and again just before each is read).  A host-fed step
+// of 256 requests: 5311 -> 1957 us (1530 us for the attention's HBM bytes
+// alone); with 4, 12 and 20 SMs 2113, 1971 and 2026 us.
+constexpr int kLinkCtas = 8;
+constexpr int kLinkGroups = 8;  // row groups per CTA (1024 threads)
+constexpr int kLinkClaim = 4;
+
+__global__ void __launch_bounds__(kLinkGroups *kRowThreads, 1) score_rows_link_kernel(
+    const uint16_t *__restrict__ ls, const uint16_t *__restrict__ lt, int vocab, int K,
+    RowOut *__restrict__ out, const NeededRows nr, int num_reqs, int max_span,
+    unsigned *__restrict__ next) {
+  extern __shared__ __align__(16) uint8_t link_smem[];
+  __shared__ unsigned s_claim[kLinkGroups];
+  const int group = threadIdx.x / kRowThreads, tid = threadIdx.x % kRowThreads;
+  const int lane = tid & 31;
+  RowSmem &sm = reinterpret_cast<RowSmem *>(link_smem)[group];
+  auto sync = [group] { named_bar_sync(1 + group, kRowThreads); };
+  const unsigned total = 2u * (unsigned)num_reqs * (unsigned)max_span;
+  for (;;) {
+    // the counter starts where the transition bounds do (kTransStart)
+    if (tid == 0) s_claim[group] = atomicAdd(next, (unsigned)kLinkClaim) - kTransStart;
+    sync();
+    const unsigned first = s_claim[group];
+    sync();  // read before the next claim overwrites it
+    if (first >= total) break;
+    // lane i < kLinkClaim holds index first + i (in every warp)
+    NeededPos mine{};
+    const unsigned i = first + lane, row = i % (2u * num_reqs), pos = i / (2u * num_reqs);
+    const bool have = lane < kLinkClaim && i < total && needed_pos(nr, num_reqs, row, pos, &mine);
+    unsigned left = __ballot_sync(0xffffffffu, have);
+    while (left) {  // the same in all four warps
+      if (tid < 32) {
+        const bool mark = (left >> lane) & 1u, open = mark && needed_now(nr, mine);
+        if (mark && !open) out[2 * mine.t + mine.model].skipped = 1;
+        const unsigned m = __ballot_sync(0xffffffffu, open);
+        if (lane == 0) s_claim[group] = m;
+      }
+      sync();
+      left = s_claim[group];
+      sync();
+      if (!left) break;
+      const int src = __ffs(left) - 1;
+      left &= left - 1;
+      NeededPos np;
+      np.r = __shfl_sync(0xffffffffu, mine.r, src);
+      np.pos = __shfl_sync(0xffffffffu, mine.pos, src);
+      np.t = __shfl_sync(0xffffffffu, mine.t, src);
+      np.model = __shfl_sync(0xffffffffu, mine.model, src);
+      np.drv = __shfl_sync(0xffffffffu, mine.drv, src);
+      np.ver = __shfl_sync(0xffffffffu, mine.ver, src);
+      score_row<false, true>(sm, (np.model ? lt : ls) + (size_t)np.t * vocab, vocab, K, 0, 1, tid,
+                             out + 2 * np.t + np.model, nr, np, sync);
     }
   }
 }
@@ -455,6 +553,12 @@ __global__ void __launch_bounds__(kEpiThreads) score_epilogue_kernel(
     const bool xok = x >= 0 && x < vocab;
     if (!xok && lane == 0) ipd_set_error(&g_score_err, IPD_DEVERR_TOKEN);
     const uint16_t *rowS = ls + (size_t)t * vocab, *rowT = lt + (size_t)t * vocab;
+    // a needed-rows pass leaves the rows past the transition unread: the
+    // values that would come from them are NaN (coverage 0), and no logit is
+    // gathered for them (the rows may lie across the host link)
+    const bool skip_s = needed_rows && rows[(size_t)2 * t * parts].skipped;
+    const bool skip_t = needed_rows && rows[(size_t)(2 * t + 1) * parts].skipped;
+    const bool both = !skip_s && !skip_t;
     // each row's records, one per part: log Z = m + log s, the entropy
     // log Z - u / s, and the top-K keys, best first (lane j holds the j-th).
     // The parts' sums combine against their common maximum, and their
@@ -484,7 +588,8 @@ __global__ void __launch_bounds__(kEpiThreads) score_epilogue_kernel(
       key2[mdl] = lane < K ? kk : 0ull;
     }
     const float nan = __int_as_float(0x7fc00000);
-    const float lxS = xok ? bf16f(rowS[x]) : nan, lxT = xok ? bf16f(rowT[x]) : nan;
+    const float lxS = xok && !skip_s ? bf16f(rowS[x]) : nan;
+    const float lxT = xok && !skip_t ? bf16f(rowT[x]) : nan;
     // union support S = Top_K(pi) u Top_K(q)
     unsigned long long kS = 0ull, kT = 0ull;
     uint32_t iS = 0, iT = 0;
@@ -504,11 +609,11 @@ __global__ void __launch_bounds__(kEpiThreads) score_epilogue_kernel(
     const bool hasS = lane < K, hasT = lane < K && !dupT;
     // a = student logit, b = teacher logit, for the two union elements of this lane
     float aS = 0.f, bS = 0.f, aT = 0.f, bT = 0.f;
-    if (hasS) {
+    if (hasS && both) {
       aS = key_val(kS);
       bS = bf16f(rowT[iS]);
     }
-    if (hasT) {
+    if (hasT && both) {
       bT = key_val(kT);
       aT = bf16f(rowS[iT]);
     }
@@ -560,14 +665,9 @@ __global__ void __launch_bounds__(kEpiThreads) score_epilogue_kernel(
     }
     // |Top_K(pi) n Top_K(q)|: teacher keys also in the student's list
     const int n_common = __popc(__ballot_sync(0xffffffffu, lane < K && dupT));
-    // a needed-rows pass leaves the rows past the transition unread: the
-    // values that would come from them are NaN (coverage 0)
-    const bool skip_s = needed_rows && rows[(size_t)2 * t * parts].skipped;
-    const bool skip_t = needed_rows && rows[(size_t)(2 * t + 1) * parts].skipped;
     const bool skip_ver = drv ? skip_s : skip_t;
     if (lane == 0) {
       const float lps = lxS - logz[0], lpt = lxT - logz[1];
-      const bool both = !skip_s && !skip_t;
       logp_s[t] = both ? lps : nan;
       logp_t[t] = both ? lpt : nan;
       feedback[t] = both ? lpt - lps : nan;
@@ -761,6 +861,20 @@ extern "C" int ipd_score_span(const uint16_t *logits_student, const uint16_t *lo
                            stream);
 }
 
+namespace {
+constexpr int kLinkSmem = kLinkGroups * (int)sizeof(RowSmem);
+
+// page-locked host memory (managed memory migrates and counts as the device's)
+bool in_host_memory(const void *p) {
+  cudaPointerAttributes a;
+  if (cudaPointerGetAttributes(&a, p) != cudaSuccess) {
+    (void)cudaGetLastError();
+    return false;
+  }
+  return a.type == cudaMemoryTypeHost;
+}
+}  // namespace
+
 extern "C" int ipd_score_span_needed(const uint16_t *logits_student,
                                      const uint16_t *logits_teacher, const int32_t *tokens,
                                      const int32_t *cu_span, const uint8_t *driver,
@@ -792,6 +906,24 @@ extern "C" int ipd_score_span_needed(const uint16_t *logits_student,
   RowOut *rows = static_cast<RowOut *>(workspace);
   int *trans = reinterpret_cast<int *>(static_cast<char *>(workspace) +
                                        trans_offset(num_reqs, total_tokens, vocab));
+  // Logits in host memory: the pass that leaves most SMs alone, unless all of
+  // its rows would start at once there too (below).
+  const bool link = total_tokens > kLinkCtas * kLinkGroups / 2 &&
+                    2LL * num_reqs * max_span <= INT32_MAX && in_host_memory(logits_student) &&
+                    in_host_memory(logits_teacher);
+  if (link) {
+    if (cudaFuncSetAttribute(score_rows_link_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             kLinkSmem) != cudaSuccess)
+      return IPD_ERR_CUDA;
+    // the bounds and, behind them, the row counter
+    if (cudaMemsetAsync(trans, 0x7f, ((size_t)num_reqs + 1) * sizeof(int), st) != cudaSuccess)
+      return IPD_ERR_CUDA;
+    score_rows_link_kernel<<<kLinkCtas, kLinkGroups * kRowThreads, kLinkSmem, st>>>(
+        logits_student, logits_teacher, vocab, K, rows,
+        NeededRows{tokens, cu_span, driver, trans, total_tokens}, num_reqs, max_span,
+        reinterpret_cast<unsigned *>(trans + num_reqs));
+    if (cudaGetLastError() != cudaSuccess) return IPD_ERR_CUDA;
+  }
   // When every row CTA fits one wave, every row starts before any transition
   // is known: the full pass (rows in up to four parts) is then as fast or
   // faster, and defines every position.
@@ -800,7 +932,7 @@ extern "C" int ipd_score_span_needed(const uint16_t *logits_student,
   const bool one_wave = cudaGetDevice(&dev) == cudaSuccess && dev >= 0 && dev < 64 &&
                         g_sms[dev] > 0 &&
                         2LL * total_tokens <= (long long)kRowCtasPerSm * g_sms[dev];
-  if (one_wave) {
+  if (one_wave && !link) {
     if (total_tokens > 0) {
       score_rows_kernel<false, false><<<2 * parts * total_tokens, kRowThreads, 0, st>>>(
           logits_student, logits_teacher, vocab, K, parts, rows, NeededRows{});
@@ -815,8 +947,8 @@ extern "C" int ipd_score_span_needed(const uint16_t *logits_student,
         max_span, false);
     return cudaGetLastError() == cudaSuccess ? IPD_OK : IPD_ERR_CUDA;
   }
-  if (total_tokens > 0) {
-    // every bound starts above any position (0x7f7f7f7f)
+  if (total_tokens > 0 && !link) {
+    // every bound starts above any position (kTransStart)
     if (cudaMemsetAsync(trans, 0x7f, (size_t)num_reqs * sizeof(int), st) != cudaSuccess)
       return IPD_ERR_CUDA;
     score_rows_kernel<false, true><<<dim3(2 * num_reqs, max_span), kRowThreads, 0, st>>>(

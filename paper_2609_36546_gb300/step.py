@@ -288,7 +288,8 @@ class VerifyStep:
         host_logits=True (needed-rows steps only, with pinned logits the
         device can read in place): the logits are not copied at all; the
         vocabulary pass reads its rows from host memory, so only the rows the
-        verdict and the emitted positions need cross the host link."""
+        verdict and the emitted positions need cross the host link.  It takes
+        a few SMs, and the attention runs on the others beside it."""
         if host_logits:
             if self.rows != "needed":
                 raise ValueError("host_logits needs a step with rows='needed'")
@@ -350,10 +351,12 @@ class VerifyStep:
             self._in.buf.copy_(host["_arena"], non_blocking=True)
         meta = torch.cuda.Event()
         meta.record(main)
-        self.run_attention(main)
+        # the vocabulary pass first: it holds a few SMs for as long as the link
+        # takes, and the attention runs on the others beside it
         sc.wait_event(meta)
         self._score_call(host["logits_s"], host["logits_t"], self.tokens, self.cu_span,
                          self.driver, self.prefix_len, self.score, sc)
+        self.run_attention(main)
         main.wait_stream(sc)
         self.run_loss(main)
         with torch.cuda.stream(main):

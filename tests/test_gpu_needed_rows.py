@@ -155,6 +155,39 @@ def test_needed_rows_from_host_equals_direct_calls(lib, graph):
     assert lib.device_error() == 0
 
 
+@pytest.mark.parametrize("n_req,span,vocab,K", [
+    (1, (70, 70), 2048, 16),      # one request, more positions than one claim
+    (33, (1, 1), 1024, 32),       # the fewest rows the link pass takes (66)
+    (40, (0, 3), 8, 8),           # empty spans, one vector a row
+    (130, (1, 17), 1040, 5),      # claims that straddle positions, ragged ends
+])
+def test_rows_over_the_host_link_match_the_resident_pass(lib, n_req, span, vocab, K):
+    """Logits in pinned host memory take the link pass; the verdict is the
+    resident full pass's, and the values agree where they are defined (the
+    full pass may sum a row in parts)."""
+    spec = S.small_spec(n_req=n_req, ctx=(80, 120), span=span, vocab=vocab, K=K, force="mixed")
+    w, step = _step(spec, 53, "all")
+    first = {k: v.cpu() for k, v in step.score.items()}
+    em, dec = _defined(step, first)
+    hs, ht = step.logits_s.cpu().pin_memory(), step.logits_t.cpu().pin_memory()
+    if not (lib.device_readable(hs) and lib.device_readable(ht)):
+        pytest.skip("pinned host memory is not mapped for the device here")
+    step.ws_score.random_(0, 255)  # whatever an earlier call left
+    for v in step.score.values():
+        v.zero_()
+    lib.score_span_needed(hs, ht, step.tokens, step.cu_span, step.driver, step.prefix_len, K, -1,
+                          step.max_span, step.score, step.ws_score)
+    torch.cuda.synchronize()
+    assert lib.device_error() == 0
+    got = {k: v.cpu() for k, v in step.score.items()}
+    for n in SCORE_REQ + ("source",):
+        assert torch.equal(got[n], first[n]), n
+    for n in ("logp_s", "logp_t", "feedback", "kl_rev", "kl_fwd"):
+        assert torch.allclose(got[n][em], first[n][em], rtol=1e-5, atol=1e-5), n
+    for n in ("covered", "margin"):
+        assert torch.equal(got[n][dec], first[n][dec]), n
+
+
 def test_host_fed_step_reading_logits_in_place(lib):
     """run_from_host(host_logits=True): the vocabulary pass reads the pinned
     host logits in place (the device copies are zeroed first, so any use of
