@@ -127,6 +127,53 @@ IPD_DEVINL float warp_sum(float v) {
   return v;
 }
 
+// Programmatic dependent launch: a kernel launched with launch_dependent may
+// start before the kernel ahead of it in the stream has finished; it calls
+// dependency_wait before it touches anything that kernel (or one before it,
+// unless that was complete when it started) writes.  Every thread of such a
+// kernel executes the wait, so its own completion implies the other's.
+// Used between the kernels of one call only; the first kernel of a call is
+// launched in full stream order.
+IPD_DEVINL void dependency_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
+// Lets the dependent kernel's blocks start once every block of this one has
+// called it (or exited).
+IPD_DEVINL void dependents_may_start() {
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
+template <typename... Params, typename... Args>
+inline cudaError_t launch_dependent(void (*kernel)(Params...), dim3 grid, dim3 block, size_t smem,
+                                    cudaStream_t st, Args &&...args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kernel, static_cast<Params>(args)...);
+}
+
+// The last r in [0, n) with cu[r] <= t (0 if there is none), found by a whole
+// warp: 32 probes at a time, so two rounds of loads up to 1024 entries where a
+// bisection by every thread takes ten in sequence.
+IPD_DEVINL int warp_find_request(const int32_t *__restrict__ cu, int n, int t) {
+  const int lane = threadIdx.x & 31;
+  int lo = 0, len = n;
+  while (len > 1) {
+    const int step = (len + 31) / 32, i = lane * step;
+    const bool le = i < len && (i == 0 || cu[lo + i] <= t);
+    const int k = 31 - __clz(__ballot_sync(0xffffffffu, le));  // lane 0 always votes
+    lo += k * step;
+    len = min(step, len - k * step);
+  }
+  return lo;
+}
+
 static constexpr float kLog2e = 1.4426950408889634f;
 static constexpr float kLn2 = 0.6931471805599453f;
 

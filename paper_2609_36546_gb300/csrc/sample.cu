@@ -307,6 +307,7 @@ __global__ void __launch_bounds__(kSampleThreads, 4) sample_partial_kernel(
   __shared__ const uint16_t *s_row[2];
   __shared__ uint32_t s_draw[2][2];
   __shared__ float s_thr[2];
+  dependency_wait();  // the verdict, when the draw follows one
   const long long nv = vocab >> 3;  // vectors per row
   const long long total = nv * n_rows;
   const long long lo = total * blockIdx.x / gridDim.x, hi = total * (blockIdx.x + 1) / gridDim.x;
@@ -364,6 +365,7 @@ __global__ void __launch_bounds__(256) sample_finalize_kernel(
     const unsigned long long *__restrict__ partial, int n_rows, int vocab, int grid,
     int32_t *__restrict__ tokens) {
   const int r = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+  dependency_wait();  // the CTAs' partials
   if (r >= n_rows) return;
   unsigned long long b = 0ull;
   if (partial) {
@@ -422,14 +424,14 @@ extern "C" __attribute__((visibility("hidden"))) int ipd_internal_sample_after_v
     grid = sample_grid(num_reqs);
     if (grid < 0) return IPD_ERR_CUDA;
     partial = static_cast<unsigned long long *>(ws);
-    sample_partial_kernel<<<grid, kSampleThreads, 0, st>>>(
-        1, ls, lt, vocab, num_reqs, philox_keys(seed), draw_base,
-        inv_temperature, cu_span, prefix_len, n_emit, next_driver, done, partial);
-    if (cudaGetLastError() != cudaSuccess) return IPD_ERR_CUDA;
+    if (launch_dependent(sample_partial_kernel, grid, kSampleThreads, 0, st, 1, ls, lt, vocab,
+                         num_reqs, philox_keys(seed), draw_base, inv_temperature, cu_span,
+                         prefix_len, n_emit, next_driver, done, partial) != cudaSuccess)
+      return IPD_ERR_CUDA;
   }
-  sample_finalize_kernel<<<(num_reqs + 7) / 8, 256, 0, st>>>(partial, num_reqs, vocab, grid,
-                                                              next_token);
-  if (cudaGetLastError() != cudaSuccess) return IPD_ERR_CUDA;
+  if (launch_dependent(sample_finalize_kernel, (num_reqs + 7) / 8, 256, 0, st, partial, num_reqs,
+                       vocab, grid, next_token) != cudaSuccess)
+    return IPD_ERR_CUDA;
   return IPD_OK;
 }
 
@@ -459,7 +461,8 @@ extern "C" int ipd_sample(const uint16_t *logits, int n_rows, int vocab, uint64_
       0, logits, nullptr, vocab, n_rows, philox_keys(seed), draw_id,
       inv_temperature, nullptr, nullptr, nullptr, nullptr, nullptr, partial);
   if (cudaGetLastError() != cudaSuccess) return IPD_ERR_CUDA;
-  sample_finalize_kernel<<<(n_rows + 7) / 8, 256, 0, st>>>(partial, n_rows, vocab, grid, tokens);
-  if (cudaGetLastError() != cudaSuccess) return IPD_ERR_CUDA;
+  if (launch_dependent(sample_finalize_kernel, (n_rows + 7) / 8, 256, 0, st, partial, n_rows, vocab,
+                       grid, tokens) != cudaSuccess)
+    return IPD_ERR_CUDA;
   return IPD_OK;
 }

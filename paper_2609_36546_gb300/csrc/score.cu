@@ -25,7 +25,7 @@ namespace {
 
 constexpr int kRowThreads = 128;  // eight row CTAs per SM: every row of a step in flight at once
 constexpr int kRowWarps = kRowThreads / 32;
-constexpr int kEpiThreads = 256;
+constexpr int kEpiThreads = 512;  // at most; a warp per span position of the request
 constexpr int kMaxParts = 4;  // a logits row is split into up to this many parts, one CTA each
 constexpr int kRowCtasPerSm = 8;  // resident row CTAs per SM (the kernel's launch bounds)
 constexpr int kMaxGroups = 32;    // group maxima a row thread keeps
@@ -525,10 +525,16 @@ __global__ void __launch_bounds__(kEpiThreads) score_epilogue_kernel(
     const int32_t *__restrict__ tokens, const int32_t *__restrict__ cu_span,
     const uint8_t *__restrict__ driver, const int32_t *__restrict__ prefix_len, int vocab, int K,
     int eos_id, const RowOut *__restrict__ rows, int parts, float *logp_s, float *logp_t,
-    float *feedback,
-    float *kl_rev, float *kl_fwd, uint8_t *covered, float *margin, uint8_t *source,
+    float *feedback, float *kl_rev, float *kl_fwd, uint8_t *covered, float *margin, uint8_t *source,
     int32_t *first_trans, int32_t *n_emit, uint8_t *next_driver, int32_t *new_len, uint8_t *done,
-    int total_tokens, const EpiOpts opt, int max_span = 0, bool needed_rows = false) {
+    int total_tokens, const EpiOpts opt, int max_span, bool needed_rows) {
+  dependency_wait();  // the row pass
+  // Latency bounds it: six dependent hops through memory and a few hundred
+  // instructions a position.  So every position has a warp of its own (up to 16
+  // to a CTA), the parts' records load side by side, the verdict is taken by a
+  // warp with ballots (one thread walked it position by position before), and
+  // the launch overlaps the row pass's end.  77 requests of up to 12 positions:
+  // 14.8 -> 12.4 us; 512 of 4: 16.9 -> 14.0 us.
   // No shared memory.  In a step that forks the vocabulary pass onto its
   // own stream, this kernel's CTAs take the SMs that the first attention
   // CTAs to finish leave free, so it runs inside the attention's tail.
@@ -548,7 +554,8 @@ __global__ void __launch_bounds__(kEpiThreads) score_epilogue_kernel(
     return;
   }
 
-  for (int t = t0 + warp; t < t1; t += kEpiThreads / 32) {
+  const int n_warps = blockDim.x >> 5;
+  for (int t = t0 + warp; t < t1; t += n_warps) {
     const int x = tokens[t];
     const bool xok = x >= 0 && x < vocab;
     if (!xok && lane == 0) ipd_set_error(&g_score_err, IPD_DEVERR_TOKEN);
@@ -569,19 +576,31 @@ __global__ void __launch_bounds__(kEpiThreads) score_epilogue_kernel(
 #pragma unroll
     for (int mdl = 0; mdl < 2; ++mdl) {
       const RowOut *pr = rows + (size_t)(2 * t + mdl) * parts;
-      float M = pr->m, S = pr->s, Uw = pr->u;
-      unsigned long long kk = pr->keys[lane];  // 0 past the part's K keys
-      for (int q = 1; q < parts; ++q) {
-        const float mq = pr[q].m, sq = pr[q].s, uq = pr[q].u;
-        const float mn = fmaxf(M, mq);
+      // every part's record in flight at once
+      float pm[kMaxParts], ps[kMaxParts], pu[kMaxParts];
+      unsigned long long pk[kMaxParts];
+#pragma unroll
+      for (int q = 0; q < kMaxParts; ++q)
+        if (q < parts) {
+          pm[q] = pr[q].m;
+          ps[q] = pr[q].s;
+          pu[q] = pr[q].u;
+          pk[q] = pr[q].keys[lane];  // 0 past the part's K keys
+        }
+      float M = pm[0], S = ps[0], Uw = pu[0];
+      unsigned long long kk = pk[0];
+#pragma unroll
+      for (int q = 1; q < kMaxParts; ++q) {
+        if (q >= parts) break;
+        const float mn = fmaxf(M, pm[q]);
         if (mn != -INFINITY) {
           const float a = M == -INFINITY ? 0.f : exp2f((M - mn) * kLog2e);
-          const float b = mq == -INFINITY ? 0.f : exp2f((mq - mn) * kLog2e);
-          S = S * a + sq * b;
-          Uw = Uw * a + uq * b;
+          const float b = pm[q] == -INFINITY ? 0.f : exp2f((pm[q] - mn) * kLog2e);
+          S = S * a + ps[q] * b;
+          Uw = Uw * a + pu[q] * b;
           M = mn;
         }
-        kk = warp_top32_u64(kk, pr[q].keys[lane], lane);
+        kk = warp_top32_u64(kk, pk[q], lane);
       }
       logz[mdl] = M + logf(S);
       ent[mdl] = logz[mdl] - Uw / S;  // H = log Z - E[l]
@@ -680,41 +699,41 @@ __global__ void __launch_bounds__(kEpiThreads) score_epilogue_kernel(
       if (opt.topk_overlap) opt.topk_overlap[t] = (float)n_common / (float)K;
     }
   }
-  __syncthreads();  // the block's writes of `covered` are visible to thread 0
-  if (threadIdx.x == 0) {
-    // Eq. (ipd_state_transition) applied position by position until the first
-    // state change or an accepted EOS; rollback rules of the verdict stage.
-    int n = 0, ft = k, nd = drv, dn = 0;
-    for (int i = 0; i < k; ++i) {
-      const int c = covered[t0 + i];
-      const bool eos = eos_id >= 0 && tokens[t0 + i] == eos_id;
-      if (drv == 0) {
-        if (!c) {  // takeover: the student token is rejected, not emitted
-          ft = i;
-          nd = 1;
-          break;
+  __syncthreads();  // the block's writes of `covered` are visible to warp 0
+  if (warp == 0) {
+    // Eq. (ipd_state_transition) up to the first state change or an accepted
+    // EOS, 32 positions at a time; rollback rules of the verdict stage.  A
+    // rejected student token (takeover) is not emitted; a teacher token is
+    // always kept, also the one after which it hands back.
+    int n = k, ft = k, nd = drv, dn = 0;
+    for (int i0 = 0; i0 < k; i0 += 32) {
+      const int i = i0 + lane;
+      const bool c = i < k && covered[t0 + i] != 0;
+      const bool eos = i < k && eos_id >= 0 && tokens[t0 + i] == eos_id;
+      const bool change = i < k && (drv == 0 ? !c : c);
+      const unsigned chg = __ballot_sync(0xffffffffu, change);
+      const unsigned stop = chg | __ballot_sync(0xffffffffu, eos);
+      if (stop) {
+        const int j = __ffs(stop) - 1;
+        const bool changed = (chg >> j) & 1u;
+        const bool rejected = changed && drv == 0;
+        n = i0 + j + (rejected ? 0 : 1);
+        if (changed) {
+          ft = i0 + j;
+          nd = 1 - drv;
         }
-        n = i + 1;
-        if (eos) {
-          dn = 1;
-          break;
-        }
-      } else {
-        n = i + 1;  // a teacher token is always kept
-        if (c) {    // handback
-          ft = i;
-          nd = 0;
-        }
-        if (eos) dn = 1;
-        if (c || eos) break;
+        dn = !rejected && __shfl_sync(0xffffffffu, (int)eos, j);
+        break;
       }
     }
-    for (int i = 0; i < k; ++i) source[t0 + i] = i < n ? (uint8_t)drv : (uint8_t)255;
-    first_trans[r] = ft;
-    n_emit[r] = n;
-    next_driver[r] = (uint8_t)nd;
-    new_len[r] = prefix_len[r] + n;
-    done[r] = (uint8_t)dn;
+    for (int i = lane; i < k; i += 32) source[t0 + i] = i < n ? (uint8_t)drv : (uint8_t)255;
+    if (lane == 0) {
+      first_trans[r] = ft;
+      n_emit[r] = n;
+      next_driver[r] = (uint8_t)nd;
+      new_len[r] = prefix_len[r] + n;
+      done[r] = (uint8_t)dn;
+    }
   }
 }
 
@@ -757,6 +776,12 @@ int row_parts(int total_tokens, int vocab, int max_parts) {
   for (int q = max_parts; q > 1; q >>= 1)
     if (2LL * total_tokens * q <= slots && vocab / 8 / q >= kRowThreads * 4) return q;
   return 1;
+}
+
+// Threads of an epilogue CTA: a warp for each of its request's positions, up to
+// 16; four where spans are short.
+int epi_threads(int num_reqs, int total_tokens) {
+  return total_tokens <= 4LL * num_reqs ? 128 : kEpiThreads;
 }
 
 // the needed-rows pass's transition bounds, after the row records and the
@@ -832,10 +857,11 @@ extern "C" int ipd_score_span_ex(const uint16_t *logits_student, const uint16_t 
           logits_student, logits_teacher, vocab, K, parts, rows, NeededRows{});
     if (cudaGetLastError() != cudaSuccess) return IPD_ERR_CUDA;
   }
-  score_epilogue_kernel<<<num_reqs, kEpiThreads, 0, st>>>(
+  launch_dependent(
+      score_epilogue_kernel, num_reqs, epi_threads(num_reqs, total_tokens), 0, st,
       logits_student, logits_teacher, tokens, cu_span, driver, prefix_len, vocab, K, eos_id, rows,
       parts, logp_s, logp_t, feedback, kl_rev, kl_fwd, covered, margin, source, first_trans,
-      n_emit, next_driver, new_len, done, total_tokens, opt);
+      n_emit, next_driver, new_len, done, total_tokens, opt, 0, false);
   if (cudaGetLastError() != cudaSuccess) return IPD_ERR_CUDA;
   if (ext && ext->next_token)
     return ipd_internal_sample_after_verdict(
@@ -938,7 +964,8 @@ extern "C" int ipd_score_span_needed(const uint16_t *logits_student,
           logits_student, logits_teacher, vocab, K, parts, rows, NeededRows{});
       if (cudaGetLastError() != cudaSuccess) return IPD_ERR_CUDA;
     }
-    score_epilogue_kernel<<<num_reqs, kEpiThreads, 0, st>>>(
+    launch_dependent(
+      score_epilogue_kernel, num_reqs, epi_threads(num_reqs, total_tokens), 0, st,
         logits_student, logits_teacher, tokens, cu_span, driver, prefix_len, vocab, K, eos_id,
         rows, parts, logp_s, logp_t, feedback, kl_rev, kl_fwd, covered, margin, source,
         first_trans, n_emit, next_driver, new_len, done, total_tokens,
@@ -956,7 +983,8 @@ extern "C" int ipd_score_span_needed(const uint16_t *logits_student,
         NeededRows{tokens, cu_span, driver, trans, total_tokens});
     if (cudaGetLastError() != cudaSuccess) return IPD_ERR_CUDA;
   }
-  score_epilogue_kernel<<<num_reqs, kEpiThreads, 0, st>>>(
+  launch_dependent(
+      score_epilogue_kernel, num_reqs, epi_threads(num_reqs, total_tokens), 0, st,
       logits_student, logits_teacher, tokens, cu_span, driver, prefix_len, vocab, K, eos_id, rows,
       1, logp_s, logp_t, feedback, kl_rev, kl_fwd, covered, margin, source, first_trans, n_emit,
       next_driver, new_len, done, total_tokens,
@@ -1252,11 +1280,13 @@ extern "C" int ipd_score_span_static(const uint16_t *logits_student,
         logits_student, logits_teacher, vocab, K, parts, rows, NeededRows{});
     if (cudaGetLastError() != cudaSuccess) return IPD_ERR_CUDA;
   }
-  score_epilogue_kernel<<<num_reqs, kEpiThreads, 0, s>>>(
+  launch_dependent(
+      score_epilogue_kernel, num_reqs, epi_threads(num_reqs, total_tokens), 0, s,
       logits_student, logits_teacher, tokens, cu_span, driver, prefix_len, vocab, K, eos_id, rows,
       parts, logp_s, logp_t, feedback, kl_rev, kl_fwd, covered, margin, source, first_trans,
       n_emit, next_driver, new_len, done, total_tokens,
-      EpiOpts{IPD_RULE_TOPK, IPD_RULE_TOPK, 0.f, 0.f, nullptr, nullptr, nullptr});
+      EpiOpts{IPD_RULE_TOPK, IPD_RULE_TOPK, 0.f, 0.f, nullptr, nullptr, nullptr, nullptr, nullptr},
+      0, false);
   if (cudaGetLastError() != cudaSuccess) return IPD_ERR_CUDA;
   return IPD_OK;
 }

@@ -130,3 +130,38 @@ def test_full_kl_matches_oracle(lib, V, T):
         assert abs(rev[t].item() - r_ref) <= FKL_ATOL + FKL_RTOL * abs(r_ref), (t, rev[t].item(), r_ref)
         assert abs(fwd[t].item() - f_ref) <= FKL_ATOL + FKL_RTOL * abs(f_ref), (t, fwd[t].item(), f_ref)
     assert rev[0].item() == 0.0 and fwd[0].item() == 0.0
+
+
+@pytest.mark.parametrize("drv", [0, 1])
+def test_verdict_of_long_spans(lib, drv):
+    """The verdict is taken 32 positions at a time: transitions and EOS at and
+    around those boundaries, both drivers, against the oracle."""
+    V, K, eos = 64, 4, 7
+    stops = [0, 1, 30, 31, 32, 33, 62, 63, 64, 65, 200]
+    cases = [(k, a, b) for k in (31, 33, 66) for a in stops for b in (200, a, 32)]
+    spans = np.array([c[0] for c in cases])
+    cu = np.concatenate([[0], np.cumsum(spans)]).astype(np.int32)
+    T, R = int(cu[-1]), len(cases)
+    g = torch.Generator().manual_seed(drv)
+    ls = torch.randn(T, V, generator=g).to(torch.bfloat16)
+    lt = torch.randn(T, V, generator=g).to(torch.bfloat16)
+    tokens = torch.randint(8, V, (T,), generator=g, dtype=torch.int32)
+    ver = ls if drv else lt
+    for r, (k, change, at_eos) in enumerate(cases):
+        for i in range(k):
+            t = int(cu[r]) + i
+            if i == at_eos:
+                tokens[t] = eos
+            covered = (i == change) if drv else (i != change)
+            ver[t, int(tokens[t])] = 30.0 if covered else -30.0
+    driver = np.full(R, drv, dtype=np.uint8)
+    prefix = np.arange(R, dtype=np.int32)
+    d = lambda a: torch.as_tensor(a).cuda()
+    out = lib.alloc_score_outputs(R, T, "cuda")
+    ws = torch.empty(lib.score_workspace_size(R, T, V, K), device="cuda", dtype=torch.uint8)
+    lib.score_span(d(ls), d(lt), d(tokens), d(cu), d(driver), d(prefix), K, eos, out, ws)
+    torch.cuda.synchronize()
+    assert lib.device_error() == 0
+    o = O.score_span(u16(ls), u16(lt), tokens.numpy(), cu, driver, prefix, K, eos)
+    for n in ("first_trans", "n_emit", "next_driver", "new_len", "done", "source"):
+        assert np.array_equal(out[n].cpu().numpy().astype(np.int64), o[n].astype(np.int64)), n

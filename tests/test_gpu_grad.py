@@ -179,3 +179,33 @@ def test_grad_full_vocabulary_rows(lib):
               1.0, (torch.float32, torch.bfloat16))
     assert (g["src"] == O.SRC_STUDENT).any() and (g["src"] == O.SRC_TEACHER).any()
     _check(g, ls, lt, K)
+
+
+def test_dense_gradient_in_place_over_the_logits(lib):
+    """grad_dense may be the student's logits themselves (the dense kernel then
+    waits for the sparse one instead of starting beside it); the result is the
+    gradient written elsewhere.  More requests than one search round holds,
+    empty spans among them."""
+    spec = S.small_spec(n_req=70, ctx=(20, 60), span=(0, 5), vocab=4096, sigma=2.5, force="mixed")
+    w = S.make_workload(spec, seed=5, device="cuda")
+    T, V, K, R = w.total_tokens, 4096, w.spec.K, 70
+    ls, lt = w.logits_s, w.logits_t
+    cu, drv, pre = w.cu_span.cuda(), w.driver.cuda(), w.prefix_len.cuda()
+    out = lib.alloc_score_outputs(R, T, "cuda")
+    ws = torch.empty(lib.score_workspace_size(R, T, V, K), device="cuda", dtype=torch.uint8)
+    tks = torch.empty((T, K), device="cuda", dtype=torch.int32)
+    tkt = torch.empty_like(tks)
+    out8 = torch.empty(8, device="cuda")
+    lib.score_span_ex(ls, lt, w.tokens, cu, drv, pre, K, -1, out, ws, topk_s=tks, topk_t=tkt)
+    lib.split_loss(out["kl_rev"], out["kl_fwd"], out["source"], cu, out["n_emit"], None, 0, 0, out8)
+    dense = torch.empty((T, V), device="cuda", dtype=torch.bfloat16)
+    gi = torch.empty((T, 2 * K), device="cuda", dtype=torch.int32)
+    gv = torch.empty((T, 2 * K), device="cuda")
+    args = (lt, tks, tkt, out["source"], cu, out["n_emit"], None, out8, K, 0, 0, 1.0, gi, gv)
+    lib.split_loss_grad(ls, *args, dense)
+    inplace = ls.clone()
+    lib.split_loss_grad(inplace, *args, inplace)
+    torch.cuda.synchronize()
+    assert lib.device_error() == 0
+    assert int((out["source"] != 255).sum()) > 20
+    assert torch.equal(inplace.view(torch.int16), dense.view(torch.int16))
