@@ -98,13 +98,25 @@ constexpr int kThreads = (kCW + 4) * 32;           // three warpgroups; warps 10
 constexpr int kRegsLaunch = 168, kRegsAux = 56, kRegsCompute = 224;
 static_assert(2 * 128 * kRegsCompute + 128 * kRegsAux <= kThreads * kRegsLaunch,
               "the register split must fit the registers the block was launched with");
-constexpr int kTargetItemsPerSm = 4;               // items of about a quarter of an SM's share
+// Items of about a quarter of an SM's share, or of half of it when a share is
+// short: a split item costs about 4 us beyond its stream (partial rows, a
+// fence, a count, the merge), a quarter of a share of 800 pages streams in 36.
+// Items of a half against a quarter, us a call: 16 requests of up to 8000 tokens,
+// 8-token spans, 355 pages a share, 97.8 / 114.5; 32 decodes of up to 4000,
+// 178 pages, 60.0 / 66.2; 32 requests of up to 16,000, 16-token spans, 1580 pages,
+// 392.8 / 377.5.
+constexpr int kTargetItemsPerSm = 4, kTargetItemsShort = 2;
+constexpr int kShortShare = 800;  // pages
 constexpr int kSizesPerBatch = 32;                // claim order: batch by batch, and within a
 constexpr int kSizeBuckets = IPD_MAX_BATCHES * kSizesPerBatch;  // batch the longest items first
 static_assert(kSizeBuckets % 32 == 0, "bucket prefix: whole lanes");
 constexpr int kMaxTargetItems = 4096;            // bound used for workspace sizing
 constexpr int kMinChunkPages = 16;
-constexpr int kSplitMax = 16;
+constexpr int kMergeBatch = 8;                   // splits of a merged row in flight at a time
+constexpr int kSplitMax = 16;                    // splits of a task; a launch
+constexpr int kSplitMaxSmall = 32;               // of few rows may split further (its partials stay small)
+constexpr long long kSmallPartialRows = 65536;   // 32 splits of every row within this many partial rows
+constexpr int kOneWaveReqs = 64;                 // requests of a launch tried for one item per SM
 constexpr int kPStride = 132;                     // floats per partial row: o[128], m, l, pad
 constexpr uint32_t kTmemCols = 512;
 // TMEM columns: the S double buffer at 0 and 128 (fp32, one column per key)
@@ -166,15 +178,16 @@ struct AttnParams {
   float scale_log2;
   int *ctrl;       // [0] n_items, [1] dynamic item counter, [2] n_tasks, [3] partial rows,
                    // [4] 1 if some task is split (claim the next item late)
-  int4 *reqinfo;   // per flattened request: (unused), task offset, partial offset, n_split
+  int4 *reqinfo;   // per flattened request: task offset, partial offset, n_split, (unused)
   Item *items;
   int *split_done; // per task: split items finished (the planner zeroes those of split tasks)
   int2 *reqslot;   // per flattened request: slot offsets of its full-size and last splits
   float *partials;
   int item_cap, task_cap;
   long long prow_cap;
-  int target_items;  // work-list size the planner aims for (a multiple of the SM count)
+  int split_max;     // most splits of a task (at most 32: one partial per lane of a merging warp)
   int n_sms;
+  int grid;          // CTAs of the attention kernel; CTA i starts with item i
 };
 
 struct StageMeta {
@@ -192,7 +205,7 @@ struct StageMeta {
 // --------------------------------------------------------------------------
 struct WsLayout {
   size_t off_ctrl, off_reqinfo, off_reqslot, off_items, off_done, off_partials, total;
-  int item_cap, task_cap, total_reqs;
+  int item_cap, task_cap, total_reqs, split_max;
   long long prow_cap;
 };
 
@@ -256,8 +269,10 @@ WsLayout layout(const ipd_attn_batch *const *bs, int n) {
     reqs += b->num_reqs;
   }
   const long long item_cap = task_cap + 2LL * kMaxTargetItems;
+  const bool small = kSplitMaxSmall * rows_all <= kSmallPartialRows;
+  L.split_max = small ? kSplitMaxSmall : kSplitMax;
   const long long prow_cap =
-      std::min<long long>(2LL * kMaxTargetItems * kTcRows, (long long)kSplitMax * rows_all);
+      std::min<long long>(2LL * kMaxTargetItems * kTcRows, (long long)L.split_max * rows_all);
   L.item_cap = (int)std::min<long long>(item_cap, 1LL << 30);
   L.task_cap = (int)std::min<long long>(task_cap, 1LL << 30);
   L.prow_cap = prow_cap;
@@ -317,31 +332,29 @@ __device__ ReqShape req_shape(const AttnParams &p, int b, int r) {
   return s;
 }
 
-template <typename T>
-__device__ T block_sum(T v, T *red) {
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  __syncthreads();
-  if (lane == 0) red[w] = v;
-  __syncthreads();
-  T t = 0;
-  for (int i = 0; i < nw; ++i) t += red[i];
-  __syncthreads();
-  return t;
-}
+// What the first pass over the requests adds up: pages over all tasks, tasks,
+// and the longest request's pages.
+struct PlanTotals {
+  long long pages;
+  int tasks, longest;
+};
 
-// maximum of one int per thread across the block (red: one slot per warp)
-__device__ int block_max_int(int v, long long *red) {
+__device__ PlanTotals block_totals(PlanTotals v, PlanTotals *red) {
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v = max(v, __shfl_xor_sync(0xffffffffu, v, o));
-  __syncthreads();
+  for (int o = 16; o > 0; o >>= 1) {
+    v.pages += __shfl_xor_sync(0xffffffffu, v.pages, o);
+    v.tasks += __shfl_xor_sync(0xffffffffu, v.tasks, o);
+    v.longest = max(v.longest, __shfl_xor_sync(0xffffffffu, v.longest, o));
+  }
   if (lane == 0) red[w] = v;
   __syncthreads();
-  int t = 0;
-  for (int i = 0; i < nw; ++i) t = max(t, (int)red[i]);
-  __syncthreads();
+  PlanTotals t{0, 0, 0};
+  for (int i = 0; i < nw; ++i) {
+    t.pages += red[i].pages;
+    t.tasks += red[i].tasks;
+    t.longest = max(t.longest, red[i].longest);
+  }
   return t;
 }
 
@@ -373,14 +386,14 @@ __device__ void block_scan4(int4 v, int4 &excl, int4 &tot, int4 *sh) {
 
 // Pages per split of a request with `pages` pages, for a target chunk size:
 // a whole number of stages, so only a request's last split ends mid-stage.
-__device__ __forceinline__ int split_pages(int pages, int chunk) {
+__device__ __forceinline__ int split_pages(int pages, int chunk, int split_max) {
   int ns = (int)(((unsigned)pages + (unsigned)chunk - 1u) / (unsigned)chunk);
-  if (ns > kSplitMax) ns = kSplitMax;
+  if (ns > split_max) ns = split_max;
   const int per = (int)(((unsigned)pages + (unsigned)ns - 1u) / (unsigned)ns);
   return (per + kStagePages - 1) / kStagePages * kStagePages;
 }
-__device__ __forceinline__ int split_count(int pages, int chunk) {
-  const int per = split_pages(pages, chunk);
+__device__ __forceinline__ int split_count(int pages, int chunk, int split_max) {
+  const int per = split_pages(pages, chunk, split_max);
   return (pages + per - 1) / per;
 }
 
@@ -433,9 +446,10 @@ constexpr int kPlanCache = 4;
 
 template <int kT>
 __global__ void __launch_bounds__(kT) attn_plan_kernel(const __grid_constant__ AttnParams p) {
-  __shared__ long long red[32];
+  __shared__ PlanTotals red[32];
   __shared__ int4 sh4[32];
-  __shared__ int s_fail;
+  __shared__ int s_fail, s_one_wave;
+  __shared__ int s_pages[kOneWaveReqs], s_tasks[kOneWaveReqs];  // of the first requests
   __shared__ int s_slot[kSizeBuckets];  // items per size bucket, then each bucket's next slot
   const int tid = threadIdx.x;
   if (tid == 0) s_fail = 0;
@@ -466,25 +480,51 @@ __global__ void __launch_bounds__(kT) attn_plan_kernel(const __grid_constant__ A
   };
   const int n_rounds = (p.total_reqs + kT - 1) / kT;
 
-  long long w = 0;
-  int pmax = 0;
+  PlanTotals mine{0, 0, 0};
   for (int k = 0; k < n_rounds; ++k) {
     const int gi = tid + k * kT;
     if (gi < p.total_reqs) {
       int b;
       const ReqShape s = shape_of(k, gi, b);
-      w += (long long)s.pages * p.b[b].hkv * s.nrb;
-      pmax = max(pmax, s.pages);
+      const int tasks = p.b[b].hkv * s.nrb;
+      mine.pages += (long long)s.pages * tasks;
+      mine.tasks += tasks;
+      mine.longest = max(mine.longest, s.pages);
+      if (gi < kOneWaveReqs) {
+        s_pages[gi] = s.pages;
+        s_tasks[gi] = tasks;
+      }
     }
   }
-  const long long W = block_sum<long long>(w, red);
-  const int P_max = block_max_int(pmax, red);
-  // chunks of a quarter of an SM's share split the long tasks for balance;
-  // when no task reaches half a share, tasks stay whole (splitting them only
-  // adds item boundaries and merges: measured 3 % on 768 tasks of <= 512
+  const PlanTotals all = block_totals(mine, red);
+  const long long W = all.pages;
+  const int P_max = all.longest;
+  // chunks of a quarter (half) of an SM's share split the long tasks for
+  // balance; when no task reaches two chunks, tasks stay whole (splitting them
+  // only adds item boundaries and merges: measured 3 % on 768 tasks of <= 512
   // pages over 152 SMs)
-  long long chunk_ll = (W + p.target_items - 1) / p.target_items;
+  const long long share = (W + p.n_sms - 1) / p.n_sms;
+  const int per_sm = share < kShortShare ? kTargetItemsShort : kTargetItemsPerSm;
+  const int target = min(kMaxTargetItems, per_sm * p.n_sms);
+  long long chunk_ll = (W + target - 1) / target;
   if ((long long)P_max <= 2 * chunk_ll) chunk_ll = P_max > chunk_ll ? P_max : chunk_ll;
+  // A short launch of fewer tasks than SMs: one item per SM if some chunk of up
+  // to 1.3 shares cuts the tasks into no more items than that (8 decodes of up to
+  // 16,000 tokens: 57.3 -> 51.9 us; 4 requests of up to 8000, 4-token spans:
+  // 57.6 -> 44.0).
+  if (share < kShortShare && p.total_reqs <= kOneWaveReqs && all.tasks <= p.n_sms) {
+    if (tid < 32) {
+      const int c = max(kMinChunkPages, (int)(share + share * tid / 100));
+      int n = 0;
+      for (int i = 0; i < p.total_reqs; ++i)
+        n += s_tasks[i] * split_count(max(s_pages[i], 1), c, p.split_max);
+      const unsigned fit = __ballot_sync(0xffffffffu, n <= p.n_sms);
+      const int best = __shfl_sync(0xffffffffu, c, fit ? __ffs(fit) - 1 : 0);
+      if (tid == 0) s_one_wave = fit ? best : 0;
+    }
+    __syncthreads();
+    if (s_one_wave) chunk_ll = s_one_wave;
+  }
   if (chunk_ll < kMinChunkPages) chunk_ll = kMinChunkPages;
   if (chunk_ll > (1LL << 30)) chunk_ll = 1LL << 30;
   const int chunk = (int)chunk_ll;
@@ -502,8 +542,8 @@ __global__ void __launch_bounds__(kT) attn_plan_kernel(const __grid_constant__ A
       int b;
       const ReqShape s = shape_of(k, gi, b);
       if (s.pages > 0) {
-        nsplit = split_count(s.pages, chunk);
-        const int per = split_pages(s.pages, chunk);
+        nsplit = split_count(s.pages, chunk, p.split_max);
+        const int per = split_pages(s.pages, chunk, p.split_max);
         const int hkv = p.b[b].hkv;
         const int tasks = hkv * s.nrb;
         cnt = make_int4(0, tasks, nsplit > 1 ? nsplit * hkv * s.rows : 0, tasks * nsplit);
@@ -517,11 +557,12 @@ __global__ void __launch_bounds__(kT) attn_plan_kernel(const __grid_constant__ A
     }
     const int off_main = warp_reserve(s_slot, bk_main, n_main);
     const int off_last = warp_reserve(s_slot, bk_last, n_last);
-    if (gi < p.total_reqs) p.reqslot[gi] = make_int2(off_main, off_last);
     int4 ex, tot;
     block_scan4(cnt, ex, tot, sh4);
-    if (gi < p.total_reqs)
-      p.reqinfo[gi] = make_int4(carry.x + ex.x, carry.y + ex.y, carry.z + ex.z, nsplit);
+    if (gi < p.total_reqs) {
+      p.reqslot[gi] = make_int2(off_main, off_last);
+      p.reqinfo[gi] = make_int4(carry.y + ex.y, carry.z + ex.z, nsplit, 0);
+    }
     carry.x += tot.x; carry.y += tot.y; carry.z += tot.z; carry.w += tot.w;
   }
   __syncthreads();
@@ -554,7 +595,7 @@ __global__ void __launch_bounds__(kT) attn_plan_kernel(const __grid_constant__ A
       s_fail = 1;
     }
     p.ctrl[0] = s_fail ? 0 : carry.w;
-    p.ctrl[1] = 0;
+    p.ctrl[1] = p.grid;  // the first item of every CTA is its own
     p.ctrl[2] = carry.y;
     p.ctrl[3] = carry.z;
     p.ctrl[4] = chunk < P_max ? 1 : 0;
@@ -562,41 +603,49 @@ __global__ void __launch_bounds__(kT) attn_plan_kernel(const __grid_constant__ A
   __syncthreads();
   if (s_fail) return;
 
+  // the items: `tpr` threads per request (a power of two): a few long requests
+  // have over a hundred items each, which one thread took 10 us to write
+  int tpr = 1;
+  while (tpr < 32 && 2 * tpr * p.total_reqs <= kT) tpr *= 2;
   for (int k = 0; k < n_rounds; ++k) {
-    const int gi = tid + k * kT;
+    const int gi = tpr > 1 ? tid / tpr : tid + k * kT;
     if (gi >= p.total_reqs) continue;
     int b;
-    const ReqShape s = shape_of(k, gi, b);
+    ReqShape s;
+    if (tpr > 1) {  // (one round)
+      b = find_batch(p, gi);
+      s = req_shape(p, b, gi - p.req_base[b]);
+    } else {
+      s = shape_of(k, gi, b);
+    }
     if (s.pages == 0) continue;
     const int r = gi - p.req_base[b];
     const int4 info = p.reqinfo[gi];
-    const int task = info.y;
-    const int ns = info.w;
-    const int per = split_pages(s.pages, chunk);
-    const int hkv = p.b[b].hkv;
-    const int tasks = hkv * s.nrb;
+    const int ns = info.z;
+    const int per = split_pages(s.pages, chunk, p.split_max);
+    const int tasks = p.b[b].hkv * s.nrb;
     const int2 rs = p.reqslot[gi];
     const int base_main = ns > 1 ? s_slot[size_bucket(b, p.n_batches, per, chunk)] + rs.x : 0;
     const int base_last =
         s_slot[size_bucket(b, p.n_batches, s.pages - (ns - 1) * per, chunk)] + rs.y;
     const int path = s.rows < kTcMinRows ? kPathCc : -1;
-    for (int sp = 0; sp < ns; ++sp) {
-      const int lo = sp * per, hi = min(s.pages, (sp + 1) * per);
-      int slot = sp < ns - 1 ? base_main + sp * tasks : base_last;
-      int task_t = task;
-      for (int kvh = 0; kvh < hkv; ++kvh) {
-        for (int rb = 0; rb < s.nrb; ++rb) {
-          const int rows = min(s.rpb, s.rows - rb * s.rpb);
-          const int pbase = ns > 1 ? info.z + ns * (kvh * s.rows + rb * s.rpb) : -1;
-          const int pth = path >= 0 ? path : tc_path(rows);
-          int4 *dst = reinterpret_cast<int4 *>(p.items + slot);
-          dst[0] = make_int4(b, r, kvh, rb);
-          dst[1] = make_int4(sp, ns, lo, hi);
-          if (ns > 1 && sp == 0) p.split_done[task_t] = 0;
-          dst[2] = make_int4(task_t++, pbase, rows, pth);
-          ++slot;
-        }
+    // split sp's items follow one another, one per task (kv head, row block)
+    int sp = 0;
+    for (int t = tid & (tpr - 1);; t += tpr) {
+      while (t >= tasks && sp < ns) {
+        t -= tasks;
+        ++sp;
       }
+      if (sp >= ns) break;
+      const int kvh = s.nrb == 1 ? t : t / s.nrb, rb = s.nrb == 1 ? 0 : t % s.nrb;
+      const int rows = min(s.rpb, s.rows - rb * s.rpb);
+      const int pbase = ns > 1 ? info.y + ns * (kvh * s.rows + rb * s.rpb) : -1;
+      const int slot = (sp < ns - 1 ? base_main + sp * tasks : base_last) + t;
+      int4 *dst = reinterpret_cast<int4 *>(p.items + slot);
+      dst[0] = make_int4(b, r, kvh, rb);
+      dst[1] = make_int4(sp, ns, sp * per, min(s.pages, (sp + 1) * per));
+      dst[2] = make_int4(info.x + t, pbase, rows, path >= 0 ? path : tc_path(rows));
+      if (ns > 1 && sp == 0) p.split_done[info.x + t] = 0;
     }
   }
 }
@@ -614,22 +663,26 @@ __device__ void merge_split_row(const AttnParams &p, const Item &I, int r, int l
   const float *base = p.partials + (size_t)(I.pbase + r) * kPStride;
   const float mv = lane < ns ? __ldcg(base + lane * sstr + 128) : -INFINITY;
   const float lv = lane < ns ? __ldcg(base + lane * sstr + 129) : 0.f;
-  float4 ov[kSplitMax];
-#pragma unroll
-  for (int sp = 0; sp < kSplitMax; ++sp)
-    if (sp < ns) ov[sp] = __ldcg(reinterpret_cast<const float4 *>(base + sp * sstr) + lane);
   const float Mx = warp_max(mv);
   const float f = mv == -INFINITY ? 0.f : ex2_approx(mv - Mx);
   const float Ls = warp_sum(lv * f);
   float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll 1
+  for (int s0 = 0; s0 < ns; s0 += kMergeBatch) {
+    float4 ov[kMergeBatch];
 #pragma unroll
-  for (int sp = 0; sp < kSplitMax; ++sp) {
-    if (sp < ns) {
-      const float fs = __shfl_sync(0xffffffffu, f, sp);
-      acc.x = fmaf(ov[sp].x, fs, acc.x);
-      acc.y = fmaf(ov[sp].y, fs, acc.y);
-      acc.z = fmaf(ov[sp].z, fs, acc.z);
-      acc.w = fmaf(ov[sp].w, fs, acc.w);
+    for (int sp = 0; sp < kMergeBatch; ++sp)
+      if (s0 + sp < ns)
+        ov[sp] = __ldcg(reinterpret_cast<const float4 *>(base + (s0 + sp) * sstr) + lane);
+#pragma unroll
+    for (int sp = 0; sp < kMergeBatch; ++sp) {
+      if (s0 + sp < ns) {
+        const float fs = __shfl_sync(0xffffffffu, f, s0 + sp);
+        acc.x = fmaf(ov[sp].x, fs, acc.x);
+        acc.y = fmaf(ov[sp].y, fs, acc.y);
+        acc.z = fmaf(ov[sp].z, fs, acc.z);
+        acc.w = fmaf(ov[sp].w, fs, acc.w);
+      }
     }
   }
   const float inv = Ls > 0.f ? 1.f / Ls : 0.f;
@@ -1681,6 +1734,7 @@ __global__ void __launch_bounds__(kThreads, 1) attn_kernel(const __grid_constant
   // the 128-byte swizzle atoms of TMA and tcgen05 assume 1024-byte alignment
   if (smem_u32(smem) & 1023u) {
     if (threadIdx.x == 0) ipd_set_error(&g_attn_err, IPD_DEVERR_PLAN);
+    dependency_wait();
     return;
   }
   if (threadIdx.x == 0) {
@@ -1704,10 +1758,15 @@ __global__ void __launch_bounds__(kThreads, 1) attn_kernel(const __grid_constant
     tc_alloc(&misc[0], kTmemCols);
     tc_relinquish();
   }
+  if (warp == kProducerWarp && lane < p.n_batches) {
+    prefetch_tensormap(&p.tmap[2 * p.b[lane].cache]);
+    prefetch_tensormap(&p.tmap[2 * p.b[lane].cache + 1]);
+  }
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = misc[0];
+  dependency_wait();  // the planner's work list
   const int n_items = p.ctrl[0];
 
   if (warp >= kCW) {
@@ -1760,14 +1819,14 @@ __global__ void __launch_bounds__(kThreads, 1) attn_kernel(const __grid_constant
       const BatchDev &Bp = p.b[I.b];
       return __ldg(Bp.page_table + (long long)I.r * Bp.max_pages + pg);
     };
-    int idx = claim();
+    int idx = blockIdx.x;  // the CTA's first item is its own
     Item I{};
     int ids = -1;
+    const bool late_claim = p.ctrl[4] != 0;
     if (idx < n_items) {
       I = p.items[idx];
       ids = load_ids(I, 0);
     }
-    const bool late_claim = p.ctrl[4] != 0;
     while (idx < n_items) {
       int nxt = n_items;
       Item In = I;
@@ -2203,8 +2262,9 @@ int launch(const ipd_attn_batch *const *bs, int n, float scale, void *ws, size_t
   P.item_cap = W.item_cap;
   P.task_cap = W.task_cap;
   P.prow_cap = W.prow_cap;
-  P.target_items = std::min(kMaxTargetItems, kTargetItemsPerSm * D.sms);
+  P.split_max = W.split_max;
   P.n_sms = D.sms;
+  P.grid = std::max(1, std::min(D.sms, W.item_cap));
 
   // a small planner block fits beside row-pass CTAs already on an SM, so a
   // step that runs both at once does not hold the attention back
@@ -2213,7 +2273,6 @@ int launch(const ipd_attn_batch *const *bs, int n, float scale, void *ws, size_t
   else
     attn_plan_kernel<kPlanThreads><<<1, kPlanThreads, 0, stream>>>(P);
   if (cudaGetLastError() != cudaSuccess) return IPD_ERR_CUDA;
-  const int grid = std::max(1, std::min(D.sms, W.item_cap));
   const bool timed = g_timing.on && g_timing.n < 4096;
   if (timed) {
     cudaEvent_t *e = &g_timing.ev[2 * g_timing.n];
@@ -2222,7 +2281,8 @@ int launch(const ipd_attn_batch *const *bs, int n, float scale, void *ws, size_t
         cudaEventRecord(e[0], stream) != cudaSuccess)
       return IPD_ERR_CUDA;
   }
-  attn_kernel<<<grid, kThreads, Smem::total, stream>>>(P);
+  if (launch_dependent(attn_kernel, P.grid, kThreads, Smem::total, stream, P) != cudaSuccess)
+    return IPD_ERR_CUDA;
   if (timed) {
     if (cudaEventRecord(g_timing.ev[2 * g_timing.n + 1], stream) != cudaSuccess)
       return IPD_ERR_CUDA;

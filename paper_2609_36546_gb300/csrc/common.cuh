@@ -192,6 +192,11 @@ IPD_DEVINL void tma_load_4d(void *dst_smem, const void *tmap, int x, int y, int 
       : "memory");
 }
 
+// Fetches a tensor map ahead of its first use.
+IPD_DEVINL void prefetch_tensormap(const void *tmap) {
+  asm volatile("prefetch.tensormap [%0];" ::"l"(tmap) : "memory");
+}
+
 // Orders this thread's generic-proxy shared-memory writes before later
 // async-proxy reads (tcgen05.mma operands written by threads).
 IPD_DEVINL void fence_proxy_async_smem() {

@@ -53,6 +53,13 @@ SMALL = [
                                        span=(2, 6)), 16),
     ("K32-ties-across-parts", S.small_spec(n_req=4, K=32, vocab=16384, sigma=2.0,
                                            tie_quantum=0.25, span=(1, 5)), 17),
+    # few requests: tasks split more than 16 ways and merged in several batches of
+    # splits, one item per SM; the most requests that are tried for that, and one more
+    ("one-long-request", S.small_spec(n_req=1, ctx=(7000, 7000), span=(5, 5)), 20),
+    ("two-long-requests", S.small_spec(n_req=2, ctx=(3000, 9000), span=(1, 3), direction="T"), 21),
+    ("one-wave-of-items", S.small_spec(n_req=9, ctx=(100, 4000), span=(1, 9)), 22),
+    ("64-sub-requests", S.small_spec(n_req=32, ctx=(1, 400), span=(1, 2), vocab=512), 23),
+    ("66-sub-requests", S.small_spec(n_req=33, ctx=(1, 400), span=(0, 2), vocab=512), 24),
 ]
 
 
