@@ -1,6 +1,6 @@
 """Compile libipd.so in-tree for sm_103a (nvcc; one translation unit per .cu,
 compiled in parallel, linked into a shared library with the CUDA runtime
-linked statically)."""
+linked statically), and the Python binding's extension module beside it."""
 from __future__ import annotations
 
 import concurrent.futures as cf
@@ -8,11 +8,13 @@ import os
 import shutil
 import subprocess
 import sys
+import sysconfig
 
 HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 OUT_DIR = os.path.join(HERE, "_lib")
 LIB = os.path.join(OUT_DIR, "libipd.so")
+NATIVE = os.path.join(OUT_DIR, "_ipd_native.so")
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 FLAGS = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", "-Xcompiler", "-Wall",
          "--expt-relaxed-constexpr"]
@@ -40,13 +42,14 @@ def _defines():
 def build(verbose: bool = False, force: bool = False) -> str:
     os.makedirs(OUT_DIR, exist_ok=True)
     srcs = sources()
-    deps = srcs + [os.path.join(CSRC, f) for f in os.listdir(CSRC) if f.endswith(".cuh")] + \
+    native_src = os.path.join(CSRC, "native.cpp")
+    deps = srcs + [native_src] + [os.path.join(CSRC, f) for f in os.listdir(CSRC) if f.endswith(".cuh")] + \
         [os.path.join(HERE, "..", "include", "ipd.h")]
     defines = _defines()
     stamp = os.path.join(OUT_DIR, "defines.txt")
     same_defines = os.path.exists(stamp) and open(stamp).read() == " ".join(defines)
-    if not force and same_defines and os.path.exists(LIB):
-        t = os.path.getmtime(LIB)
+    if not force and same_defines and os.path.exists(LIB) and os.path.exists(NATIVE):
+        t = os.path.getmtime(NATIVE)  # written last
         if all(os.path.getmtime(d) <= t for d in deps):
             return LIB
     nvcc = _nvcc()
@@ -71,6 +74,15 @@ def build(verbose: bool = False, force: bool = False) -> str:
     if r.returncode != 0:
         raise RuntimeError(f"link failed:\n{r.stdout}\n{r.stderr}")
     os.replace(tmp, LIB)
+    # the extension links against the library in its own folder
+    tmp = NATIVE + ".tmp"
+    r = subprocess.run(["g++", "-O2", "-std=c++17", "-Wall", "-fPIC", "-shared", "-fvisibility=hidden",
+                        "-I", sysconfig.get_paths()["include"], native_src, "-o", tmp,
+                        "-L", OUT_DIR, "-l:libipd.so", "-Wl,-rpath,$ORIGIN"],
+                       capture_output=True, text=True)
+    if r.returncode != 0:
+        raise RuntimeError(f"the binding's extension failed to build:\n{r.stdout}\n{r.stderr}")
+    os.replace(tmp, NATIVE)
     with open(stamp, "w") as f:
         f.write(" ".join(defines))
     return LIB

@@ -1,13 +1,17 @@
-"""ctypes binding of libipd.so: argument marshalling only.
+"""Binding of libipd.so: argument marshalling only.
 
 Every function here forwards torch tensors (device memory) as raw pointers to
 the C ABI declared in include/ipd.h and raises IpdError on a non-zero status.
-No step of the computation runs in Python, and there is no fallback: if the
-shared library cannot be loaded, importing the binding fails.
+The calls a step issues are marshalled by a small extension module
+(csrc/native.cpp); queries and settings go through ctypes.  No step of the
+computation runs in Python, and there is no fallback: if the shared library or
+the extension cannot be loaded, importing the binding fails.
 """
 from __future__ import annotations
 
 import ctypes
+import importlib.machinery
+import importlib.util
 import os
 from typing import Optional, Sequence
 
@@ -15,6 +19,7 @@ import torch
 
 _HERE = os.path.dirname(os.path.abspath(__file__))
 LIB_PATH = os.path.join(_HERE, "_lib", "libipd.so")
+NATIVE_PATH = os.path.join(_HERE, "_lib", "_ipd_native.so")
 
 IPD_OK = 0
 STATUS = {0: "IPD_OK", 1: "IPD_ERR_INVALID_ARG", 2: "IPD_ERR_UNSUPPORTED", 3: "IPD_ERR_WORKSPACE",
@@ -54,7 +59,16 @@ def _load():
     return ctypes.CDLL(LIB_PATH)
 
 
+def _load_native():
+    loader = importlib.machinery.ExtensionFileLoader("_ipd_native", NATIVE_PATH)
+    spec = importlib.util.spec_from_file_location("_ipd_native", NATIVE_PATH, loader=loader)
+    mod = importlib.util.module_from_spec(spec)
+    loader.exec_module(mod)
+    return mod
+
+
 _lib = _load()
+_native = _load_native()
 
 c_p = ctypes.c_void_p
 c_i = ctypes.c_int
@@ -155,6 +169,8 @@ def _ptr(t: Optional[torch.Tensor]) -> Optional[int]:
 
 def _stream(stream) -> Optional[int]:
     if stream is None:
+        if torch.cuda.is_initialized():  # the current stream's handle, without a Stream object
+            return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
         return torch.cuda.current_stream().cuda_stream if torch.cuda.is_available() else None
     return stream.cuda_stream if hasattr(stream, "cuda_stream") else int(stream)
 
@@ -212,19 +228,13 @@ def attn_workspace_size(verify: Sequence[AttnBatch], decode: Sequence[AttnBatch]
 
 def verify_attn(verify: Sequence[AttnBatch], decode: Sequence[AttnBatch], softmax_scale: float,
                 workspace: torch.Tensor, stream=None):
-    va, nv = _arr(verify)
-    da, nd = _arr(decode)
-    _check(_lib.ipd_verify_attn(va, nv, da, nd, softmax_scale, _ptr(workspace),
-                                workspace.numel() * workspace.element_size(), _stream(stream)),
+    _check(_native.attn(verify, decode, softmax_scale, workspace, _stream(stream)),
            "ipd_verify_attn")
 
 
 def decode_attn(decode: Sequence[AttnBatch], softmax_scale: float, workspace: torch.Tensor,
                 stream=None):
-    da, nd = _arr(decode)
-    _check(_lib.ipd_decode_attn(da, nd, softmax_scale, _ptr(workspace),
-                                workspace.numel() * workspace.element_size(), _stream(stream)),
-           "ipd_decode_attn")
+    _check(_native.attn((), decode, softmax_scale, workspace, _stream(stream)), "ipd_decode_attn")
 
 
 def score_workspace_size(num_reqs: int, total_tokens: int, vocab: int, K: int) -> int:
@@ -247,15 +257,8 @@ def alloc_score_outputs(num_reqs: int, total_tokens: int, device) -> dict:
 
 def score_span(logits_student, logits_teacher, tokens, cu_span, driver, prefix_len, K: int,
                eos_id: int, out: dict, workspace: torch.Tensor, stream=None):
-    R = driver.numel()
-    T, V = logits_student.shape
-    _check(_lib.ipd_score_span(
-        _ptr(logits_student), _ptr(logits_teacher), _ptr(tokens), _ptr(cu_span), _ptr(driver),
-        _ptr(prefix_len), R, T, V, K, eos_id,
-        *[_ptr(out[n]) for n, _ in SCORE_TOKEN_OUTPUTS],
-        *[_ptr(out[n]) for n, _ in SCORE_REQ_OUTPUTS],
-        _ptr(workspace), workspace.numel() * workspace.element_size(), _stream(stream)),
-        "ipd_score_span")
+    _check(_native.score(0, logits_student, logits_teacher, tokens, cu_span, driver, prefix_len, K,
+                         eos_id, 0, out, None, workspace, _stream(stream)), "ipd_score_span")
 
 
 def device_readable(t: torch.Tensor) -> bool:
@@ -271,15 +274,9 @@ def score_span_needed(logits_student, logits_teacher, tokens, cu_span, driver, p
                       stream=None):
     """ipd_score_span reading only the rows the verdict and the emitted
     positions need; ``max_span`` bounds every request's span length."""
-    R = driver.numel()
-    T, V = logits_student.shape
-    _check(_lib.ipd_score_span_needed(
-        _ptr(logits_student), _ptr(logits_teacher), _ptr(tokens), _ptr(cu_span), _ptr(driver),
-        _ptr(prefix_len), R, T, V, K, eos_id, max_span,
-        *[_ptr(out[n]) for n, _ in SCORE_TOKEN_OUTPUTS],
-        *[_ptr(out[n]) for n, _ in SCORE_REQ_OUTPUTS],
-        _ptr(workspace), workspace.numel() * workspace.element_size(), _stream(stream)),
-        "ipd_score_span_needed")
+    _check(_native.score(1, logits_student, logits_teacher, tokens, cu_span, driver, prefix_len, K,
+                         eos_id, max_span, out, None, workspace, _stream(stream)),
+           "ipd_score_span_needed")
 
 
 def score_span_ex(logits_student, logits_teacher, tokens, cu_span, driver, prefix_len, K: int,
@@ -296,27 +293,17 @@ def score_span_ex(logits_student, logits_teacher, tokens, cu_span, driver, prefi
     optional per-token entropies and top-K overlap ratio (fp32 [T] tensors),
     top-K id lists (int32 [T, K]) and the next span's first token per request
     (int32 [R]; draw numbers from ``draw_base``, uint64 as int64 [R])."""
-    R = driver.numel()
-    T, V = logits_student.shape
-    ext = _ScoreExt(takeover_rule, handback_rule, takeover_tau, handback_tau,
-                    _ptr(entropy_s), _ptr(entropy_t), _ptr(topk_overlap), _ptr(topk_s),
-                    _ptr(topk_t), _ptr(next_token), _ptr(draw_base),
-                    sample_seed & 0xFFFFFFFFFFFFFFFF, inv_temperature)
-    _check(_lib.ipd_score_span_ex(
-        _ptr(logits_student), _ptr(logits_teacher), _ptr(tokens), _ptr(cu_span), _ptr(driver),
-        _ptr(prefix_len), R, T, V, K, eos_id,
-        *[_ptr(out[n]) for n, _ in SCORE_TOKEN_OUTPUTS],
-        *[_ptr(out[n]) for n, _ in SCORE_REQ_OUTPUTS],
-        ctypes.byref(ext), _ptr(workspace), workspace.numel() * workspace.element_size(),
-        _stream(stream)), "ipd_score_span_ex")
+    ext = (takeover_rule, handback_rule, takeover_tau, handback_tau, entropy_s, entropy_t,
+           topk_overlap, topk_s, topk_t, next_token, draw_base, sample_seed, inv_temperature)
+    _check(_native.score(2, logits_student, logits_teacher, tokens, cu_span, driver, prefix_len, K,
+                         eos_id, 0, out, ext, workspace, _stream(stream)), "ipd_score_span_ex")
 
 
 def full_kl(logits_student, logits_teacher, kl_rev_full: torch.Tensor, kl_fwd_full: torch.Tensor,
             stream=None):
     """Full-vocabulary KL in both directions at every span position."""
-    T, V = logits_student.shape
-    _check(_lib.ipd_full_kl(_ptr(logits_student), _ptr(logits_teacher), T, V, _ptr(kl_rev_full),
-                            _ptr(kl_fwd_full), _stream(stream)), "ipd_full_kl")
+    _check(_native.full_kl(logits_student, logits_teacher, kl_rev_full, kl_fwd_full,
+                           _stream(stream)), "ipd_full_kl")
 
 
 def score_span_static(logits_student, logits_teacher, tokens, cu_span, driver, prefix_len,
@@ -324,47 +311,28 @@ def score_span_static(logits_student, logits_teacher, tokens, cu_span, driver, p
     """ipd_score_span without a workspace: for callers that cannot allocate
     device memory (the scratch is the library's static device array, at most
     STATIC_MAX_TOKENS span positions; overlapping calls race on it)."""
-    R = driver.numel()
-    T, V = logits_student.shape
-    _check(_lib.ipd_score_span_static(
-        _ptr(logits_student), _ptr(logits_teacher), _ptr(tokens), _ptr(cu_span), _ptr(driver),
-        _ptr(prefix_len), R, T, V, K, eos_id,
-        *[_ptr(out[n]) for n, _ in SCORE_TOKEN_OUTPUTS],
-        *[_ptr(out[n]) for n, _ in SCORE_REQ_OUTPUTS],
-        _stream(stream)), "ipd_score_span_static")
+    _check(_native.score(3, logits_student, logits_teacher, tokens, cu_span, driver, prefix_len, K,
+                         eos_id, 0, out, None, None, _stream(stream)), "ipd_score_span_static")
 
 
 def split_loss(kl_rev, kl_fwd, source, cu_span, n_emit, resp_len, agg_mode: int, dir_mode: int,
                out8: torch.Tensor, stream=None):
-    R = cu_span.numel() - 1
-    _check(_lib.ipd_split_loss(_ptr(kl_rev), _ptr(kl_fwd), _ptr(source), _ptr(cu_span),
-                               _ptr(n_emit), _ptr(resp_len), R, agg_mode, dir_mode, _ptr(out8),
-                               None, 0, _stream(stream)), "ipd_split_loss")
+    _check(_native.split_loss(kl_rev, kl_fwd, source, cu_span, n_emit, resp_len, agg_mode,
+                              dir_mode, out8, _stream(stream)), "ipd_split_loss")
 
 
 def kv_append(cache: "KVCache", k_new, v_new, cu_new, seq_len, page_table, stream=None):
     """Writes the new tokens' K/V rows ([n, Hkv, 128] bf16) into the cache's
     pages at the last positions of each request's sequence (``seq_len`` is
     the length after the append)."""
-    R = cu_new.numel() - 1
-    _check(_lib.ipd_kv_append(_ptr(cache.k_pages), _ptr(cache.v_pages), cache.k_pages.shape[0],
-                              cache.k_pages.shape[1], 16, 128, _ptr(k_new), _ptr(v_new),
-                              _ptr(cu_new), _ptr(seq_len), _ptr(page_table),
-                              page_table.shape[1], R, k_new.shape[0], _stream(stream)),
-           "ipd_kv_append")
+    append = (cache, k_new, v_new, cu_new, seq_len, page_table)
+    _check(_native.kv_append_many((append,), _stream(stream)), "ipd_kv_append")
 
 
 def kv_append_many(appends, stream=None):
     """Several appends in one launch: ``appends`` is a sequence of (cache,
     k_new, v_new, cu_new, seq_len, page_table) tuples, each as in kv_append."""
-    n = len(appends)
-    arr = (_KvAppendDesc * max(n, 1))()
-    for i, (cache, k_new, v_new, cu_new, seq_len, page_table) in enumerate(appends):
-        arr[i] = _KvAppendDesc(_ptr(cache.k_pages), _ptr(cache.v_pages), cache.k_pages.shape[0],
-                               cache.k_pages.shape[1], 16, 128, _ptr(k_new), _ptr(v_new),
-                               _ptr(cu_new), _ptr(seq_len), _ptr(page_table),
-                               page_table.shape[1], cu_new.numel() - 1, k_new.shape[0])
-    _check(_lib.ipd_kv_append_many(arr, n, _stream(stream)), "ipd_kv_append_many")
+    _check(_native.kv_append_many(appends, _stream(stream)), "ipd_kv_append_many")
 
 
 def sample_workspace_size(n_rows: int, vocab: int) -> int:
@@ -375,11 +343,8 @@ def sample(logits, seed: int, draw_id: Optional[torch.Tensor], tokens: torch.Ten
            workspace: torch.Tensor, inv_temperature: float = 1.0, stream=None):
     """One seeded draw per row of ``logits`` ([n, V] bf16) into ``tokens``
     (int32 [n]); ``draw_id`` holds the rows' uint64 draw numbers (as int64)."""
-    n, V = logits.shape
-    _check(_lib.ipd_sample(_ptr(logits), n, V, seed & 0xFFFFFFFFFFFFFFFF, _ptr(draw_id),
-                           inv_temperature, _ptr(tokens), _ptr(workspace),
-                           workspace.numel() * workspace.element_size(), _stream(stream)),
-           "ipd_sample")
+    _check(_native.sample(logits, seed & 0xFFFFFFFFFFFFFFFF, draw_id, tokens, workspace,
+                          inv_temperature, _stream(stream)), "ipd_sample")
 
 
 def split_loss_grad(logits_student, logits_teacher, topk_s, topk_t, source, cu_span, n_emit,
@@ -389,18 +354,15 @@ def split_loss_grad(logits_student, logits_teacher, topk_s, topk_t, source, cu_s
     """Gradient of grad_scale * loss with respect to the student's logits:
     sparse [T, 2K] ids / values, and the dense [T, V] form when ``grad_dense``
     (fp32 or bf16) is given."""
-    R = cu_span.numel() - 1
-    T, V = logits_student.shape
     dtype = DTYPE_F32
     if grad_dense is not None:
         if grad_dense.dtype == torch.bfloat16:
             dtype = DTYPE_BF16
         elif grad_dense.dtype != torch.float32:
             raise IpdError(STATUS_CODES["IPD_ERR_INVALID_ARG"], "ipd_split_loss_grad: dense dtype")
-    _check(_lib.ipd_split_loss_grad(
-        _ptr(logits_student), _ptr(logits_teacher), _ptr(topk_s), _ptr(topk_t), _ptr(source),
-        _ptr(cu_span), _ptr(n_emit), _ptr(resp_len), _ptr(loss_out8), R, T, V, K, agg_mode,
-        dir_mode, grad_scale, _ptr(grad_idx), _ptr(grad_val), _ptr(grad_dense), dtype, None, 0,
+    _check(_native.split_loss_grad(
+        logits_student, logits_teacher, topk_s, topk_t, source, cu_span, n_emit, resp_len,
+        loss_out8, K, agg_mode, dir_mode, grad_scale, grad_idx, grad_val, grad_dense, dtype,
         _stream(stream)), "ipd_split_loss_grad")
 
 

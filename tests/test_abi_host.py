@@ -233,3 +233,69 @@ def test_attn_kernel_timing_host_side():
     assert L.ipd_attn_kernel_time(ctypes.byref(ms), ctypes.byref(n)) == 0
     assert n.value == 0 and ms.value == 0.0          # nothing launched: nothing recorded
     assert L.ipd_set_attn_kernel_timing(0) == 0
+
+
+def test_binding_marshals_and_refuses(ipd):
+    """The extension module behind the step's calls: statuses come back as
+    IpdError, malformed arguments as Python errors, before anything is
+    launched (CPU tensors stand in for device memory)."""
+    z = lambda *s, dt=torch.float32: torch.zeros(s, dtype=dt)
+    bf, i32 = torch.bfloat16, torch.int32
+    with pytest.raises(ipd.IpdError) as e:
+        ipd.full_kl(z(3, 4095, dt=bf), z(3, 4095, dt=bf), z(3), z(3), stream=0)
+    assert e.value.status == ipd.STATUS_CODES["IPD_ERR_UNSUPPORTED"]
+    with pytest.raises(ValueError):
+        ipd.full_kl(z(4096, dt=bf), z(4096, dt=bf), z(1), z(1), stream=0)
+    with pytest.raises(AttributeError):
+        ipd.full_kl("logits", z(1, 8, dt=bf), z(1), z(1), stream=0)
+    with pytest.raises(ipd.IpdError) as e:
+        ipd.sample(z(2, 16, dt=bf), 1, None, z(2, dt=i32), z(8, dt=torch.uint8), 1.0, stream=0)
+    assert e.value.status == ipd.STATUS_CODES["IPD_ERR_WORKSPACE"]
+    out = ipd.alloc_score_outputs(1, 2, "cpu")
+    args = (z(2, 16, dt=bf), z(2, 16, dt=bf), z(2, dt=i32), z(2, dt=i32), z(1, dt=torch.uint8),
+            z(1, dt=i32))
+    ws = z(4, dt=torch.uint8)
+    for call, extra in ((ipd.score_span, ()), (ipd.score_span_needed, (5,)),
+                        (ipd.score_span_ex, ())):
+        for K, code in ((16, "IPD_ERR_WORKSPACE"), (33, "IPD_ERR_UNSUPPORTED")):
+            with pytest.raises(ipd.IpdError) as e:
+                call(*args, K, -1, *extra, out, ws, stream=0)
+            assert e.value.status == ipd.STATUS_CODES[code]
+    with pytest.raises(ipd.IpdError) as e:
+        ipd.score_span_static(z(5000, 8, dt=bf), z(5000, 8, dt=bf), *args[2:], 4, -1, out, stream=0)
+    assert e.value.status == ipd.STATUS_CODES["IPD_ERR_CAPACITY"]
+    with pytest.raises(ipd.IpdError) as e:
+        ipd.score_span_ex(*args, 16, -1, out, ws, takeover_rule=9, stream=0)
+    assert e.value.status == ipd.STATUS_CODES["IPD_ERR_INVALID_ARG"]
+    with pytest.raises(KeyError):
+        ipd.score_span(*args, 16, -1, {}, ws, stream=0)
+    with pytest.raises(TypeError):
+        ipd.score_span(*args, 1.5, -1, out, ws, stream=0)
+    with pytest.raises(ipd.IpdError) as e:
+        ipd.split_loss(z(2), z(2), z(2, dt=torch.uint8), z(2, dt=i32), z(1, dt=i32), None, 7, 0, z(8),
+                       stream=0)
+    assert e.value.status == ipd.STATUS_CODES["IPD_ERR_INVALID_ARG"]
+    with pytest.raises(ipd.IpdError) as e:
+        ipd.split_loss_grad(args[0], args[1], z(2, 4, dt=i32), z(2, 4, dt=i32),
+                            z(2, dt=torch.uint8), z(2, dt=i32), z(1, dt=i32), None, z(8), 4, 0, 0,
+                            float("inf"), z(2, 8, dt=i32), z(2, 8), stream=0)
+    assert e.value.status == ipd.STATUS_CODES["IPD_ERR_INVALID_ARG"]
+    cache = ipd.KVCache(z(2, 4, 16, 128, dt=bf), z(2, 4, 16, 128, dt=bf))
+    append = (cache, z(1, 4, 128, dt=bf), z(1, 4, 128, dt=bf), z(2, dt=i32), z(1, dt=i32),
+              z(1, 1, dt=i32))
+    ipd.kv_append_many([], stream=0)  # nothing to do
+    for appends, err in (([append] * 9, ipd.IpdError), ([append[:5]], ValueError)):
+        with pytest.raises(err):
+            ipd.kv_append_many(appends, stream=0)
+    batch = ipd.AttnBatch(cache, z(1, 32, 128, dt=bf), z(2, dt=i32), z(1, dt=i32), z(1, 1, dt=i32),
+                          z(1, 32, 128, dt=bf), 1, 16)
+    for batches, scale, code in (([batch] * 9, 0.1, "IPD_ERR_INVALID_ARG"),
+                                 ([batch], 0.0, "IPD_ERR_INVALID_ARG"),
+                                 ([batch], 0.1, "IPD_ERR_WORKSPACE")):
+        for call in (lambda b, s: ipd.verify_attn(b, [], s, ws, stream=0),
+                     lambda b, s: ipd.decode_attn(b, s, ws, stream=0)):
+            with pytest.raises(ipd.IpdError) as e:
+                call(batches, scale)
+            assert e.value.status == ipd.STATUS_CODES[code]
+    with pytest.raises(AttributeError):
+        ipd.verify_attn([object()], [], 0.1, ws, stream=0)
