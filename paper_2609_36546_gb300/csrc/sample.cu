@@ -37,7 +37,15 @@ namespace {
 constexpr uint32_t kPhiloxM0 = 0xD2511F53u, kPhiloxM1 = 0xCD9E8D57u;
 constexpr uint32_t kPhiloxW0 = 0x9E3779B9u, kPhiloxW1 = 0xBB67AE85u;
 constexpr uint32_t kLog2eBits = 0x3FB8AA3Bu;
+// Two CTAs an SM with two vectors of a thread in work at once: fewer warps find
+// their first threshold, longer stretches use it, and the two vectors' Philox
+// chains fill the issue slots.  192 / 1000 rows of 151,936, us a call: 34.1 / 130.9;
+// one vector at a time with four CTAs 39.2 / -, three 36.6 / 139.5, two 35.1 /
+// 136.0; two vectors with three CTAs 37.3 / 138.2, with one CTA of 512 threads
+// 45.0 / 142.5.
 constexpr int kSampleThreads = 256;
+constexpr int kSampleCtas = 2;  // resident CTAs per SM
+constexpr int kSampleVecs = 2;  // vectors of a thread worked on at once
 constexpr int kSampleGridCap = 2048;  // CTAs of one launch when the rows are fewer
 
 // The ten round keys of one seed (key + i * Weyl increment), passed by value
@@ -224,25 +232,13 @@ __device__ __forceinline__ void scan_row(const uint16_t *__restrict__ row, int v
   const int lane = threadIdx.x & 31;
   const unsigned long long c2 = f2_pack(cf, cf);
   const PhiloxRow pr = philox_row(draw_lo, draw_hi, key);
+  const uint4 *src = reinterpret_cast<const uint4 *>(row);
   int vec = v_lo + (int)threadIdx.x;
   bs = -INFINITY;
   bv = vec < v_hi ? vec * 8 : -1;
-  uint4 nxt = make_uint4(0, 0, 0, 0);
-  if (vec < v_hi) nxt = __ldg(reinterpret_cast<const uint4 *>(row) + vec);
-  for (int first = vec - lane; first < v_hi; first += kSampleThreads, vec += kSampleThreads) {
-    const uint4 raw = nxt;
-    if (vec + kSampleThreads < v_hi)
-      nxt = __ldg(reinterpret_cast<const uint4 *>(row) + vec + kSampleThreads);
-    const uint4 ra = philox10(2u * (uint32_t)vec, pr, key);
-    const uint4 rb = philox10(2u * (uint32_t)vec + 1u, pr, key);
-    // the vector's bound: its largest logit with its largest random word.  With
-    // y = 2^32 - 1 - bits, y 2^-32 is at most 2 (1 - u), so the bound needs one
-    // more unit of slack than an entry's own; y = 0 gives +inf
-    const uint32_t r8 = max(max(max(ra.x, ra.y), max(ra.z, ra.w)),
-                            max(max(rb.x, rb.y), max(rb.z, rb.w)));
-    const float b8 = __fsub_rn(__fmul_rn(bf16x8_max(raw), cf), lg2_approx(__uint2float_rn(~r8)));
-    float thr = *s_thr;
-    if (!__any_sync(0xffffffffu, vec < v_hi && b8 >= thr - 33.f)) continue;
+
+  // a vector whose bound reaches the threshold, with its random words
+  auto examine = [&](int vec, const uint4 &raw, const uint4 &ra, const uint4 &rb, float &thr) {
     // the entries' own bounds, the entry's number in the low three bits
     float ub[8];
     bound_x2(raw.x, ra.x, ra.y, c2, ub[0], ub[1]);
@@ -276,7 +272,61 @@ __device__ __forceinline__ void scan_row(const uint16_t *__restrict__ row, int v
       top = max8(rest);
     }
     if (lane == 0 && thr > *s_thr) *s_thr = thr;
+  };
+
+  uint4 nxt[kSampleVecs];
+#pragma unroll
+  for (int u = 0; u < kSampleVecs; ++u) {
+    nxt[u] = make_uint4(0, 0, 0, 0);
+    if (vec + u * kSampleThreads < v_hi) nxt[u] = __ldg(src + vec + u * kSampleThreads);
   }
+  constexpr int kStep = kSampleVecs * kSampleThreads;
+#pragma unroll 1
+  for (int first = vec - lane; first < v_hi; first += kStep, vec += kStep) {
+    uint4 raw[kSampleVecs], ra[kSampleVecs], rb[kSampleVecs];
+    float b8[kSampleVecs];
+#pragma unroll
+    for (int u = 0; u < kSampleVecs; ++u) {
+      const int v = vec + u * kSampleThreads;
+      raw[u] = nxt[u];
+      if (v + kStep < v_hi) nxt[u] = __ldg(src + v + kStep);
+      ra[u] = philox10(2u * (uint32_t)v, pr, key);
+      rb[u] = philox10(2u * (uint32_t)v + 1u, pr, key);
+      // the vector's bound: its largest logit with its largest random word.  With
+      // y = 2^32 - 1 - bits, y 2^-32 is at most 2 (1 - u), so the bound needs one
+      // more unit of slack than an entry's own; y = 0 gives +inf
+      const uint32_t r8 = max(max(max(ra[u].x, ra[u].y), max(ra[u].z, ra[u].w)),
+                              max(max(rb[u].x, rb[u].y), max(rb[u].z, rb[u].w)));
+      b8[u] = __fsub_rn(__fmul_rn(bf16x8_max(raw[u]), cf), lg2_approx(__uint2float_rn(~r8)));
+      if (v >= v_hi) b8[u] = -INFINITY;
+    }
+    float thr = *s_thr;
+    bool reach = false;
+#pragma unroll
+    for (int u = 0; u < kSampleVecs; ++u) reach |= b8[u] >= thr - 33.f;
+    if (!__any_sync(0xffffffffu, reach)) continue;
+#pragma unroll
+    for (int u = 0; u < kSampleVecs; ++u)
+      examine(vec + u * kSampleThreads, raw[u], ra[u], rb[u], thr);
+  }
+}
+
+// How the rows' vectors are cut: CTA i takes `len` of them, one more if i < rem,
+// from piece_begin(i) on.
+struct Pieces {
+  int len, rem;
+};
+__device__ __forceinline__ long long piece_begin(const Pieces &p, int i) {
+  return (long long)i * p.len + min(i, p.rem);
+}
+// a / b, in 32 bits where a fits (a 64-bit division takes over a hundred
+// instructions of every warp)
+__device__ __forceinline__ int div_small(long long a, int b) {
+  return (a >> 32) == 0 ? (int)((uint32_t)a / (uint32_t)b) : (int)(a / b);
+}
+__device__ __forceinline__ int piece_of(const Pieces &p, long long x) {
+  const long long longer = (long long)(p.len + 1) * p.rem;
+  return x < longer ? div_small(x, p.len + 1) : p.rem + div_small(x - longer, p.len);
 }
 
 // One draw per row of a list of rows.  mode 0: row r is row r of `rows0`
@@ -287,18 +337,17 @@ __device__ __forceinline__ void scan_row(const uint16_t *__restrict__ row, int v
 // draws nothing.
 //
 // Bound: the integer pipes.  Philox's 36 wide multiplies a vector keep the
-// heavy half of the FMA pipe half busy and the whole takes 24 warp
-// instructions an entry (44 when every entry was scored); the rows are read at
-// 1.5 TB/s.  192 rows of 151,936: 57.3 -> 41.3 us a call; four CTAs an SM
-// rather than five, which spilled (44.0 against 47.3 us in an earlier form).
+// heavy half of the FMA pipe over half busy, and the rows are read at 1.7 TB/s.
+// 192 rows of 151,936: 57.3 us a call with every entry scored (44 warp
+// instructions an entry), 34.1 now.
 //
 // Work split: the rows' 8-entry vectors form one flat range that is cut into
 // gridDim.x equal pieces, one per CTA (grid >= rows, so a piece meets at most
 // two rows).  Each CTA stores its best key for the first and the second row
 // it meets (0 where it meets none).
-__global__ void __launch_bounds__(kSampleThreads, 4) sample_partial_kernel(
+__global__ void __launch_bounds__(kSampleThreads, kSampleCtas) sample_partial_kernel(
     int mode, const uint16_t *__restrict__ rows0, const uint16_t *__restrict__ rows1, int vocab,
-    int n_rows, const PhiloxKeys key, const uint64_t *__restrict__ draw_id,
+    int n_rows, const Pieces pieces, const PhiloxKeys key, const uint64_t *__restrict__ draw_id,
     float inv_temperature, const int32_t *__restrict__ cu_span,
     const int32_t *__restrict__ prefix_len, const int32_t *__restrict__ n_emit,
     const uint8_t *__restrict__ next_driver, const uint8_t *__restrict__ done,
@@ -308,10 +357,9 @@ __global__ void __launch_bounds__(kSampleThreads, 4) sample_partial_kernel(
   __shared__ uint32_t s_draw[2][2];
   __shared__ float s_thr[2];
   dependency_wait();  // the verdict, when the draw follows one
-  const long long nv = vocab >> 3;  // vectors per row
-  const long long total = nv * n_rows;
-  const long long lo = total * blockIdx.x / gridDim.x, hi = total * (blockIdx.x + 1) / gridDim.x;
-  const int row_lo = (int)(lo / nv);
+  const int nv = vocab >> 3;  // vectors per row
+  const long long lo = piece_begin(pieces, blockIdx.x), hi = piece_begin(pieces, blockIdx.x + 1);
+  const int row_lo = div_small(lo, nv);
   if (threadIdx.x < 2) {
     const int r = row_lo + (int)threadIdx.x;
     const uint16_t *row = nullptr;
@@ -362,21 +410,20 @@ __global__ void __launch_bounds__(kSampleThreads, 4) sample_partial_kernel(
 // one warp per row: the best key over the CTAs whose piece meets the row ->
 // token id (-1: none)
 __global__ void __launch_bounds__(256) sample_finalize_kernel(
-    const unsigned long long *__restrict__ partial, int n_rows, int vocab, int grid,
+    const unsigned long long *__restrict__ partial, int n_rows, int vocab, const Pieces pieces,
     int32_t *__restrict__ tokens) {
   const int r = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
   dependency_wait();  // the CTAs' partials
   if (r >= n_rows) return;
   unsigned long long b = 0ull;
   if (partial) {
-    const long long nv = vocab >> 3, total = nv * n_rows;
-    // CTA i covers [floor(i total / grid), floor((i + 1) total / grid)); the
-    // CTA holding vector x is the largest i with floor(i total / grid) <= x
-    auto cta_of = [&](long long x) { return (int)(((x + 1) * grid + total - 1) / total) - 1; };
-    const int i0 = cta_of((long long)r * nv), i1 = cta_of((long long)(r + 1) * nv - 1);
+    const int nv = vocab >> 3;
+    const int i0 = piece_of(pieces, (long long)r * nv);
+    const int i1 = piece_of(pieces, (long long)(r + 1) * nv - 1);
     for (int i = i0 + lane; i <= i1; i += 32) {
-      const int first_row = (int)((total * i / grid) / nv);
-      b = max_u64(b, partial[2 * (size_t)i + (first_row == r ? 0 : 1)]);
+      // row r is the first of its CTA's two unless the piece began before it
+      const int second = piece_begin(pieces, i) < (long long)r * nv ? 1 : 0;
+      b = max_u64(b, partial[2 * (size_t)i + second]);
     }
   }
 #pragma unroll
@@ -402,6 +449,11 @@ int sample_grid(int n_rows) {
   return n_rows > cap[dev] ? n_rows : cap[dev];
 }
 
+Pieces sample_pieces(int n_rows, int vocab, int grid) {
+  const long long total = (long long)n_rows * (vocab >> 3);
+  return Pieces{(int)(total / grid), (int)(total % grid)};
+}
+
 }  // namespace
 
 extern "C" __attribute__((visibility("hidden"))) size_t ipd_internal_sample_ws(int n_rows,
@@ -425,12 +477,12 @@ extern "C" __attribute__((visibility("hidden"))) int ipd_internal_sample_after_v
     if (grid < 0) return IPD_ERR_CUDA;
     partial = static_cast<unsigned long long *>(ws);
     if (launch_dependent(sample_partial_kernel, grid, kSampleThreads, 0, st, 1, ls, lt, vocab,
-                         num_reqs, philox_keys(seed), draw_base, inv_temperature, cu_span,
+                         num_reqs, sample_pieces(num_reqs, vocab, grid), philox_keys(seed), draw_base, inv_temperature, cu_span,
                          prefix_len, n_emit, next_driver, done, partial) != cudaSuccess)
       return IPD_ERR_CUDA;
   }
   if (launch_dependent(sample_finalize_kernel, (num_reqs + 7) / 8, 256, 0, st, partial, num_reqs,
-                       vocab, grid, next_token) != cudaSuccess)
+                       vocab, sample_pieces(num_reqs, vocab, grid), next_token) != cudaSuccess)
     return IPD_ERR_CUDA;
   return IPD_OK;
 }
@@ -458,11 +510,11 @@ extern "C" int ipd_sample(const uint16_t *logits, int n_rows, int vocab, uint64_
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
   unsigned long long *partial = static_cast<unsigned long long *>(workspace);
   sample_partial_kernel<<<grid, kSampleThreads, 0, st>>>(
-      0, logits, nullptr, vocab, n_rows, philox_keys(seed), draw_id,
+      0, logits, nullptr, vocab, n_rows, sample_pieces(n_rows, vocab, grid), philox_keys(seed), draw_id,
       inv_temperature, nullptr, nullptr, nullptr, nullptr, nullptr, partial);
   if (cudaGetLastError() != cudaSuccess) return IPD_ERR_CUDA;
   if (launch_dependent(sample_finalize_kernel, (n_rows + 7) / 8, 256, 0, st, partial, n_rows, vocab,
-                       grid, tokens) != cudaSuccess)
+                       sample_pieces(n_rows, vocab, grid), tokens) != cudaSuccess)
     return IPD_ERR_CUDA;
   return IPD_OK;
 }
