@@ -1008,10 +1008,14 @@ extern "C" int ipd_score_span_needed(const uint16_t *logits_student,
 // ---------------------------------------------------------------------------
 namespace {
 constexpr int kKlThreads = 256;
-constexpr int kKlCtasPerSm = 4;  // the kernel's launch bounds
+// Bound: HBM, once enough loads are in flight (7.0 TB/s over 4000 positions).
+// A call of up to three CTAs an SM keeps twelve loads a thread in flight, larger
+// ones eight with four CTAs an SM; 333 positions of 151,936, us a call: 38.2, with
+// eight 40.4, without the loads ahead 45.0 (16 in flight spill, 45.3).
+constexpr int kKlDeepU = 3, kKlDeepCtas = 3;
 
-template <int P>
-__global__ void __launch_bounds__(kKlThreads, kKlCtasPerSm) full_kl_kernel(
+template <int P, int U, int kCtas>
+__global__ void __launch_bounds__(kKlThreads, kCtas) full_kl_kernel(
     const uint16_t *__restrict__ ls, const uint16_t *__restrict__ lt, int vocab,
     float *__restrict__ kl_rev, float *__restrict__ kl_fwd) {
   __shared__ float sh[kKlThreads / 32][6];
@@ -1026,16 +1030,27 @@ __global__ void __launch_bounds__(kKlThreads, kKlCtasPerSm) full_kl_kernel(
   float ms = -INFINITY, mt = -INFINITY;
   unsigned long long ss = 0ull, st = 0ull, aa = 0ull, bb = 0ull;  // packed pairs
   const unsigned long long l2e = f2_pack(kLog2e, kLog2e);
-  constexpr int U = 2;
+  // Each iteration takes U 16-byte vectors of each row per thread and issues
+  // the next iteration's 2 U loads before it works on them.
+  const uint4 none = make_uint4(0xff80ff80u, 0xff80ff80u, 0xff80ff80u, 0xff80ff80u);  // -inf
+  uint4 ns[U], nt[U];
+#pragma unroll
+  for (int u = 0; u < U; ++u) {
+    const int v = v_lo + u * kKlThreads + (int)threadIdx.x;
+    ns[u] = v < nvec ? ldg_stream(rs + v) : none;
+    nt[u] = v < nvec ? ldg_stream(rt + v) : none;
+  }
   for (int base = v_lo; base < nvec; base += kKlThreads * U) {
     uint4 xs[U], xt[U];
     bool ok[U];
 #pragma unroll
     for (int u = 0; u < U; ++u) {
-      const int v = base + u * kKlThreads + (int)threadIdx.x;
+      xs[u] = ns[u];
+      xt[u] = nt[u];
+      const int v = base + u * kKlThreads + (int)threadIdx.x, vn = v + U * kKlThreads;
       ok[u] = v < nvec;
-      xs[u] = ok[u] ? ldg_stream(rs + v) : make_uint4(0xff80ff80u, 0xff80ff80u, 0xff80ff80u, 0xff80ff80u);
-      xt[u] = ok[u] ? ldg_stream(rt + v) : make_uint4(0xff80ff80u, 0xff80ff80u, 0xff80ff80u, 0xff80ff80u);
+      ns[u] = vn < nvec ? ldg_stream(rs + vn) : none;
+      nt[u] = vn < nvec ? ldg_stream(rt + vn) : none;
     }
     float bs = -INFINITY, bt = -INFINITY;
 #pragma unroll
@@ -1157,11 +1172,11 @@ __global__ void __launch_bounds__(kKlThreads, kKlCtasPerSm) full_kl_kernel(
 
 int g_kl_sms[64] = {};  // SM count per device, read once
 
-template <int P>
+template <int P, int U, int kCtas>
 cudaError_t launch_full_kl(const uint16_t *ls, const uint16_t *lt, int T, int vocab, float *rev,
                            float *fwd, cudaStream_t st) {
   if (P == 1) {
-    full_kl_kernel<1><<<T, kKlThreads, 0, st>>>(ls, lt, vocab, rev, fwd);
+    full_kl_kernel<1, U, kCtas><<<T, kKlThreads, 0, st>>>(ls, lt, vocab, rev, fwd);
     return cudaGetLastError();
   }
   cudaLaunchConfig_t cfg = {};
@@ -1175,7 +1190,7 @@ cudaError_t launch_full_kl(const uint16_t *ls, const uint16_t *lt, int T, int vo
   at[0].val.clusterDim.z = 1;
   cfg.attrs = at;
   cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, full_kl_kernel<P>, ls, lt, vocab, rev, fwd);
+  return cudaLaunchKernelEx(&cfg, full_kl_kernel<P, U, kCtas>, ls, lt, vocab, rev, fwd);
 }
 }  // namespace
 
@@ -1189,27 +1204,30 @@ extern "C" int ipd_full_kl(const uint16_t *logits_student, const uint16_t *logit
     return IPD_ERR_INVALID_ARG;
   if (((uintptr_t)logits_student | (uintptr_t)logits_teacher) & 15) return IPD_ERR_INVALID_ARG;
   // parts per position: as many as keep every CTA of the call in one wave,
-  // with at least two loads per thread and row in a part
+  // with at least two loads per thread and row in a part (more parts for the
+  // sake of an even load, 666 or 1332 CTAs for 333 positions: 49.1 and 44.8 us
+  // against 40.1; clusters fill the SMs badly)
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return IPD_ERR_CUDA;
   if (!g_kl_sms[dev] &&
       cudaDeviceGetAttribute(&g_kl_sms[dev], cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
     return IPD_ERR_CUDA;
-  const long long slots = (long long)kKlCtasPerSm * g_kl_sms[dev];
+  const long long sms = g_kl_sms[dev];
   int P = 1;
   for (int q = 4; q > 1; q >>= 1)
-    if ((long long)total_tokens * q <= slots && vocab / 8 / q >= kKlThreads * 2) {
+    if ((long long)total_tokens * q <= 4 * sms && vocab / 8 / q >= kKlThreads * 2) {
       P = q;
       break;
     }
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
-  const cudaError_t e =
-      P == 4 ? launch_full_kl<4>(logits_student, logits_teacher, total_tokens, vocab, kl_rev_full,
-                                 kl_fwd_full, st)
-      : P == 2 ? launch_full_kl<2>(logits_student, logits_teacher, total_tokens, vocab,
-                                   kl_rev_full, kl_fwd_full, st)
-               : launch_full_kl<1>(logits_student, logits_teacher, total_tokens, vocab,
-                                   kl_rev_full, kl_fwd_full, st);
+  auto run = [&](auto launch) {
+    return launch(logits_student, logits_teacher, total_tokens, vocab, kl_rev_full, kl_fwd_full, st);
+  };
+  const cudaError_t e = P == 4                     ? run(launch_full_kl<4, 2, 4>)
+                        : P == 2                   ? run(launch_full_kl<2, 2, 4>)
+                        : total_tokens <= kKlDeepCtas * sms
+                            ? run(launch_full_kl<1, kKlDeepU, kKlDeepCtas>)
+                            : run(launch_full_kl<1, 2, 4>);
   if (e != cudaSuccess || cudaGetLastError() != cudaSuccess) return IPD_ERR_CUDA;
   return IPD_OK;
 }
