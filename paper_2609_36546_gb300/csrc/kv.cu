@@ -3,12 +3,17 @@
 // verifier's prefill writes the span's tokens into its cache; each happens
 // before the attention that reads them).
 //
-// One thread per 16-byte piece of a row (a 128-wide bf16 head row is 16
-// pieces): consecutive threads cover one head row, then the next head, then
-// the next token, so both the reads of the new rows and the writes into a
-// page slot are contiguous 256-byte runs.  Every write is bounds-checked
-// against the request offsets, the sequence length, the page table and the
-// pool; a bad entry is recorded in the device error word and skipped.  One launch takes up to IPD_MAX_BATCHES appends
+// One warp per new token: its K and V head rows (a 128-wide bf16 head row is
+// 16 pieces of 16 bytes) are contiguous in the inputs, and each head row is a
+// contiguous 256-byte run of a page slot.  A few microseconds of latency bound
+// the launch (a step moves a few MB), so a lane's loads, up to eight, are in
+// flight while the warp looks the token's request up in one or two rounds of
+// probes and follows the page table, once per token.  Spans of 8 of 256 requests,
+// us a call: 6.6, with a thread and a bisection per 16-byte piece 8.2; of 16 of
+// 300: 8.2 and 14.9; of 24 of 768: 25.5 and 43.1; small appends the same (6.4).
+// Every write is bounds-checked against the request offsets, the sequence
+// length, the page table and the pool; a bad entry is recorded in the device
+// error word and skipped.  One launch takes up to IPD_MAX_BATCHES appends
 // (caches and request batches), so a step's appends cost one launch.
 #include <cuda_runtime.h>
 #include <stdint.h>
@@ -21,7 +26,9 @@ IPD_DECLARE_ERROR_WORD(g_kv_err);
 namespace {
 
 constexpr int kPieces = 16;  // 16-byte pieces per 128-wide bf16 row
-constexpr int kAppendThreads = 256;
+constexpr int kAppendThreads = 128;
+constexpr int kAppendWarps = kAppendThreads / 32;
+constexpr int kAppendLoads = 8;  // pieces of a lane in flight (a token of 8 KV heads)
 
 // One append (one cache, one batch of requests) of a launch.
 struct AppendDev {
@@ -29,63 +36,73 @@ struct AppendDev {
   const uint16_t *k_new, *v_new;
   const int32_t *cu_new, *seq_len, *page_table;
   long long num_pages;
-  long long n_units;  // total_new * hkv * kPieces pieces of K (as many of V)
-  int hkv, max_pages, num_reqs, pad;
+  int total_new, hkv, max_pages, num_reqs;
 };
 
 struct AppendParams {
   AppendDev d[IPD_MAX_BATCHES];
-  long long end[IPD_MAX_BATCHES];  // exclusive prefix of 2 n_units over the appends
+  long long end[IPD_MAX_BATCHES];  // inclusive prefix of total_new over the appends
   int n;
 };
 
 __global__ void __launch_bounds__(kAppendThreads) kv_append_kernel(
     const __grid_constant__ AppendParams P) {
   const long long total = P.end[P.n - 1];
-  for (long long u0 = (long long)blockIdx.x * kAppendThreads + threadIdx.x; u0 < total;
-       u0 += (long long)gridDim.x * kAppendThreads) {
+  const int lane = threadIdx.x & 31;
+  for (long long u0 = (long long)blockIdx.x * kAppendWarps + (threadIdx.x >> 5); u0 < total;
+       u0 += (long long)gridDim.x * kAppendWarps) {
     int di = 0;
     while (di + 1 < P.n && u0 >= P.end[di]) ++di;
     const AppendDev &D = P.d[di];
-    const long long u = u0 - (di > 0 ? P.end[di - 1] : 0);
-    const bool is_v = u >= D.n_units;
-    const long long w = is_v ? u - D.n_units : u;
-    const long long per_tok = (long long)D.hkv * kPieces;
-    const int tok = (int)(w / per_tok);
-    const int rem = (int)(w % per_tok);
-    const int h = rem / kPieces, c = rem % kPieces;
+    const int tok = (int)(u0 - (di > 0 ? P.end[di - 1] : 0));
+    const int half = D.hkv * kPieces, n = 2 * half;  // pieces of K, of K and V
+    const uint4 *ks = reinterpret_cast<const uint4 *>(D.k_new) + (size_t)tok * half;
+    const uint4 *vs = reinterpret_cast<const uint4 *>(D.v_new) + (size_t)tok * half;
+    uint4 v[kAppendLoads];
+    auto load = [&](int p0) {
+#pragma unroll
+      for (int j = 0; j < kAppendLoads; ++j) {
+        const int p = p0 + 32 * j + lane;
+        if (p < n) v[j] = p < half ? ks[p] : vs[p - half];
+      }
+    };
+    load(0);
     // a row that no request's offsets cover is not written
     if (tok < D.cu_new[0] || tok >= D.cu_new[D.num_reqs]) {
-      ipd_set_error(&g_kv_err, IPD_DEVERR_SPAN);
+      if (lane == 0) ipd_set_error(&g_kv_err, IPD_DEVERR_SPAN);
       continue;
     }
-    // the request holding new row `tok`: the last r with cu_new[r] <= tok
-    int lo = 0, hi = D.num_reqs - 1;
-    while (lo < hi) {
-      const int mid = (lo + hi + 1) >> 1;
-      if (D.cu_new[mid] <= tok) lo = mid;
-      else hi = mid - 1;
-    }
-    const int n = D.cu_new[lo + 1] - D.cu_new[lo];
-    const int p = D.seq_len[lo] - n + (tok - D.cu_new[lo]);  // absolute position of the row
-    if (p < 0 || p >= D.seq_len[lo] || (p >> 4) >= D.max_pages) {
-      ipd_set_error(&g_kv_err, IPD_DEVERR_SEQ_LEN);
+    const int r = warp_find_request(D.cu_new, D.num_reqs, tok);
+    const int first = D.cu_new[r], len = D.seq_len[r];
+    const int pos = len - (D.cu_new[r + 1] - first) + (tok - first);  // absolute position of the row
+    if (pos < 0 || pos >= len || (pos >> 4) >= D.max_pages) {
+      if (lane == 0) ipd_set_error(&g_kv_err, IPD_DEVERR_SEQ_LEN);
       continue;
     }
-    const int page = D.page_table[(size_t)lo * D.max_pages + (p >> 4)];
+    const int page = D.page_table[(size_t)r * D.max_pages + (pos >> 4)];
     if (page < 0 || page >= D.num_pages) {
-      ipd_set_error(&g_kv_err, IPD_DEVERR_PAGE_ID);
+      if (lane == 0) ipd_set_error(&g_kv_err, IPD_DEVERR_PAGE_ID);
       continue;
     }
-    const uint4 *src = reinterpret_cast<const uint4 *>(is_v ? D.v_new : D.k_new);
-    uint4 *dst = reinterpret_cast<uint4 *>(is_v ? D.v_pages : D.k_pages);
-    dst[(((size_t)page * D.hkv + h) * 16 + (p & 15)) * kPieces + c] =
-        src[((size_t)tok * D.hkv + h) * kPieces + c];
+    // head 0's row of the slot; head h's is 16 rows further per head
+    const size_t slot = ((size_t)page * D.hkv * 16 + (pos & 15)) * kPieces;
+    uint4 *kd = reinterpret_cast<uint4 *>(D.k_pages) + slot;
+    uint4 *vd = reinterpret_cast<uint4 *>(D.v_pages) + slot;
+    for (int p0 = 0; p0 < n; p0 += 32 * kAppendLoads) {
+      if (p0 > 0) load(p0);
+#pragma unroll
+      for (int j = 0; j < kAppendLoads; ++j) {
+        const int p = p0 + 32 * j + lane;
+        if (p >= n) break;
+        const int q = p < half ? p : p - half;
+        (p < half ? kd : vd)[(size_t)(q / kPieces) * 16 * kPieces + q % kPieces] = v[j];
+      }
+    }
   }
 }
 
 // Host validation of one append; fills its device descriptor.  IPD_OK with
-// n_units == 0 for an append with no rows.
+// total_new == 0 for an append with no rows.
 int check_append(const ipd_kv_append_desc &a, AppendDev *d) {
   if (a.num_reqs < 0 || a.total_new < 0 || a.num_pages < 0 || a.num_kv_heads < 1 ||
       a.max_pages < 1)
@@ -100,8 +117,7 @@ int check_append(const ipd_kv_append_desc &a, AppendDev *d) {
       15)
     return IPD_ERR_INVALID_ARG;
   *d = AppendDev{a.k_pages, a.v_pages, a.k_new, a.v_new, a.cu_new, a.seq_len, a.page_table,
-                 a.num_pages, (long long)a.total_new * a.num_kv_heads * kPieces,
-                 a.num_kv_heads, a.max_pages, a.num_reqs, 0};
+                 a.num_pages, a.total_new, a.num_kv_heads, a.max_pages, a.num_reqs};
   return IPD_OK;
 }
 
@@ -114,14 +130,14 @@ int launch_appends(const ipd_kv_append_desc *descs, int n, ipd_stream_t stream) 
     AppendDev d;
     const int st = check_append(descs[i], &d);
     if (st != IPD_OK) return st;
-    if (d.n_units == 0) continue;  // nothing to write: not part of the launch
+    if (d.total_new == 0) continue;  // nothing to write: not part of the launch
     P.d[P.n] = d;
-    total += 2 * d.n_units;
+    total += d.total_new;
     P.end[P.n] = total;
     ++P.n;
   }
   if (P.n == 0) return IPD_OK;
-  const long long blocks = (total + kAppendThreads - 1) / kAppendThreads;
+  const long long blocks = (total + kAppendWarps - 1) / kAppendWarps;
   const int grid = (int)(blocks < 8192 ? blocks : 8192);
   kv_append_kernel<<<grid, kAppendThreads, 0, reinterpret_cast<cudaStream_t>(stream)>>>(P);
   if (cudaGetLastError() != cudaSuccess) return IPD_ERR_CUDA;

@@ -58,6 +58,9 @@ def _run(lib, kp, vp, kn, vn, cu, L, table):
     (4, [100, 7, 0, 31, 64], [8, 8, 8, 1, 16]),            # teacher-shaped spans, page crossings
     (8, [1000, 15, 16, 300], [1, 1, 1, 1]),                # student decode appends
     (2, [3, 50, 0], [0, 17, 33]),                          # an empty request, multi-page spans
+    (1, [9] * 1030, [0, 1, 2, 0, 0] * 206),                # three rounds of the request search
+    (1, [4] * 33, [1] * 33),                               # two rounds, the second ragged
+    (20, [3, 9], [2, 5]),                                  # more pieces than a warp's first loads
 ])
 def test_kv_append_bit_exact(lib, hkv, old_len, n_new):
     case = _case(hkv, hkv, old_len, n_new)
