@@ -219,11 +219,13 @@ class VerifyStep:
             return
         main = stream if stream is not None else torch.cuda.current_stream(self.device)
         if getattr(self, "_side", None) is None:
-            self._side = torch.cuda.Stream(device=self.device)
+            # its kernels go first where either stream's could start (8 requests
+            # of up to 4000 tokens, replayed: 77 -> 70 us; 1024 requests: 6554 -> 6393)
+            self._side = torch.cuda.Stream(device=self.device, priority=-1)
         side = self._side
         side.wait_stream(main)
-        self.run_attention(main)
         self.run_score(side)
+        self.run_attention(main)
         self.run_loss(side)
         main.wait_stream(side)
 
