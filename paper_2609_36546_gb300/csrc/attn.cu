@@ -116,7 +116,7 @@ constexpr int kMergeBatch = 8;                   // splits of a merged row in fl
 constexpr int kSplitMax = 16;                    // splits of a task; a launch
 constexpr int kSplitMaxSmall = 32;               // of few rows may split further (its partials stay small)
 constexpr long long kSmallPartialRows = 65536;   // 32 splits of every row within this many partial rows
-constexpr int kOneWaveReqs = 64;                 // requests of a launch tried for one item per SM
+constexpr int kSmallPlanReqs = 32;               // requests of a launch planned by one warp
 constexpr int kPStride = 132;                     // floats per partial row: o[128], m, l, pad
 constexpr uint32_t kTmemCols = 512;
 // TMEM columns: the S double buffer at 0 and 128 (fp32, one column per key)
@@ -332,11 +332,11 @@ __device__ ReqShape req_shape(const AttnParams &p, int b, int r) {
   return s;
 }
 
-// What the first pass over the requests adds up: pages over all tasks, tasks,
-// and the longest request's pages.
+// What the first pass over the requests finds: pages over all tasks, and the
+// longest request's pages.
 struct PlanTotals {
   long long pages;
-  int tasks, longest;
+  int longest;
 };
 
 __device__ PlanTotals block_totals(PlanTotals v, PlanTotals *red) {
@@ -344,15 +344,13 @@ __device__ PlanTotals block_totals(PlanTotals v, PlanTotals *red) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) {
     v.pages += __shfl_xor_sync(0xffffffffu, v.pages, o);
-    v.tasks += __shfl_xor_sync(0xffffffffu, v.tasks, o);
     v.longest = max(v.longest, __shfl_xor_sync(0xffffffffu, v.longest, o));
   }
   if (lane == 0) red[w] = v;
   __syncthreads();
-  PlanTotals t{0, 0, 0};
+  PlanTotals t{0, 0};
   for (int i = 0; i < nw; ++i) {
     t.pages += red[i].pages;
-    t.tasks += red[i].tasks;
     t.longest = max(t.longest, red[i].longest);
   }
   return t;
@@ -395,6 +393,19 @@ __device__ __forceinline__ int split_pages(int pages, int chunk, int split_max) 
 __device__ __forceinline__ int split_count(int pages, int chunk, int split_max) {
   const int per = split_pages(pages, chunk, split_max);
   return (pages + per - 1) / per;
+}
+
+// Pages per item before rounding: W pages over all tasks, the longest task
+// P_max.  Chunks of a quarter (half) of an SM's share split the long tasks for
+// balance; when no task reaches two chunks, tasks stay whole (splitting them
+// only adds item boundaries and merges: measured 3 % on 768 tasks of <= 512
+// pages over 152 SMs).
+__device__ __forceinline__ long long chunk_rule(const AttnParams &p, long long W, int P_max) {
+  const long long share = (W + p.n_sms - 1) / p.n_sms;
+  const int per_sm = share < kShortShare ? kTargetItemsShort : kTargetItemsPerSm;
+  const int target = min(kMaxTargetItems, per_sm * p.n_sms);
+  const long long chunk = (W + target - 1) / target;
+  return P_max <= 2 * chunk && P_max > chunk ? P_max : chunk;
 }
 
 // Claim-order bucket of an item of batch `b` with `n` pages; higher buckets
@@ -448,8 +459,7 @@ template <int kT>
 __global__ void __launch_bounds__(kT) attn_plan_kernel(const __grid_constant__ AttnParams p) {
   __shared__ PlanTotals red[32];
   __shared__ int4 sh4[32];
-  __shared__ int s_fail, s_one_wave;
-  __shared__ int s_pages[kOneWaveReqs], s_tasks[kOneWaveReqs];  // of the first requests
+  __shared__ int s_fail;
   __shared__ int s_slot[kSizeBuckets];  // items per size bucket, then each bucket's next slot
   const int tid = threadIdx.x;
   if (tid == 0) s_fail = 0;
@@ -480,51 +490,20 @@ __global__ void __launch_bounds__(kT) attn_plan_kernel(const __grid_constant__ A
   };
   const int n_rounds = (p.total_reqs + kT - 1) / kT;
 
-  PlanTotals mine{0, 0, 0};
+  PlanTotals mine{0, 0};
   for (int k = 0; k < n_rounds; ++k) {
     const int gi = tid + k * kT;
     if (gi < p.total_reqs) {
       int b;
       const ReqShape s = shape_of(k, gi, b);
-      const int tasks = p.b[b].hkv * s.nrb;
-      mine.pages += (long long)s.pages * tasks;
-      mine.tasks += tasks;
+      mine.pages += (long long)s.pages * p.b[b].hkv * s.nrb;
       mine.longest = max(mine.longest, s.pages);
-      if (gi < kOneWaveReqs) {
-        s_pages[gi] = s.pages;
-        s_tasks[gi] = tasks;
-      }
     }
   }
   const PlanTotals all = block_totals(mine, red);
   const long long W = all.pages;
   const int P_max = all.longest;
-  // chunks of a quarter (half) of an SM's share split the long tasks for
-  // balance; when no task reaches two chunks, tasks stay whole (splitting them
-  // only adds item boundaries and merges: measured 3 % on 768 tasks of <= 512
-  // pages over 152 SMs)
-  const long long share = (W + p.n_sms - 1) / p.n_sms;
-  const int per_sm = share < kShortShare ? kTargetItemsShort : kTargetItemsPerSm;
-  const int target = min(kMaxTargetItems, per_sm * p.n_sms);
-  long long chunk_ll = (W + target - 1) / target;
-  if ((long long)P_max <= 2 * chunk_ll) chunk_ll = P_max > chunk_ll ? P_max : chunk_ll;
-  // A short launch of fewer tasks than SMs: one item per SM if some chunk of up
-  // to 1.3 shares cuts the tasks into no more items than that (8 decodes of up to
-  // 16,000 tokens: 57.3 -> 51.9 us; 4 requests of up to 8000, 4-token spans:
-  // 57.6 -> 44.0).
-  if (share < kShortShare && p.total_reqs <= kOneWaveReqs && all.tasks <= p.n_sms) {
-    if (tid < 32) {
-      const int c = max(kMinChunkPages, (int)(share + share * tid / 100));
-      int n = 0;
-      for (int i = 0; i < p.total_reqs; ++i)
-        n += s_tasks[i] * split_count(max(s_pages[i], 1), c, p.split_max);
-      const unsigned fit = __ballot_sync(0xffffffffu, n <= p.n_sms);
-      const int best = __shfl_sync(0xffffffffu, c, fit ? __ffs(fit) - 1 : 0);
-      if (tid == 0) s_one_wave = fit ? best : 0;
-    }
-    __syncthreads();
-    if (s_one_wave) chunk_ll = s_one_wave;
-  }
+  long long chunk_ll = chunk_rule(p, W, P_max);
   if (chunk_ll < kMinChunkPages) chunk_ll = kMinChunkPages;
   if (chunk_ll > (1LL << 30)) chunk_ll = 1LL << 30;
   const int chunk = (int)chunk_ll;
@@ -647,6 +626,139 @@ __global__ void __launch_bounds__(kT) attn_plan_kernel(const __grid_constant__ A
       dst[2] = make_int4(info.x + t, pbase, rows, path >= 0 ? path : tc_path(rows));
       if (ns > 1 && sp == 0) p.split_done[info.x + t] = 0;
     }
+  }
+}
+
+// Planner of a launch of at most 32 requests (over all batches): one warp holds
+// a request per lane and finds the item boundaries with warp scans, where the
+// planner above meets at a dozen block barriers; then the whole block writes the
+// items.  Latency bounds it (two dependent hops through memory and the warp's
+// own instructions).  Claim order: batch by batch, the requests with the largest
+// items first, a request's splits together (16 requests of up to 8000 tokens,
+// 8-token spans: 92.2 us; in the order of the planner above 97.0, all last
+// splits at the end 102.5).
+constexpr int kSmallPlanThreads = 256;
+
+// inclusive prefix sum over the warp
+__device__ __forceinline__ int warp_prefix(int v) {
+  const int lane = threadIdx.x & 31;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const int y = __shfl_up_sync(0xffffffffu, v, o);
+    if (lane >= o) v += y;
+  }
+  return v;
+}
+
+__global__ void __launch_bounds__(kSmallPlanThreads) attn_plan_small_kernel(
+    const __grid_constant__ AttnParams p) {
+  // requests in claim order: ends of their items, first task and partial row,
+  // pages, pages per split, rows, and batch << 24 | request
+  __shared__ int s_item_end[32], s_task0[32], s_prow0[32];
+  __shared__ int s_pages[32], s_per[32], s_rows[32], s_br[32];
+  __shared__ int s_n_items;
+  const int tid = threadIdx.x, lane = tid & 31;
+  if (tid < 32) {
+    int b = 0, nrb = 0, pages = 0, rows = 0, br = 0;
+    if (lane < p.total_reqs) {
+      b = find_batch(p, lane);
+      const int r = lane - p.req_base[b];
+      const ReqShape s = req_shape(p, b, r);
+      pages = s.pages;
+      rows = s.rows;
+      nrb = s.nrb;
+      br = b << 24 | r;
+    }
+    int tasks = p.b[b].hkv * nrb;
+    long long W = (long long)pages * tasks;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) W += __shfl_xor_sync(0xffffffffu, W, o);
+    const int longest = __reduce_max_sync(0xffffffffu, pages);
+    long long chunk_ll = max((long long)kMinChunkPages, chunk_rule(p, W, longest));
+    // A short launch of fewer tasks than SMs: one item per SM if some chunk not
+    // much above the share cuts the tasks into no more items than that.  Against
+    // two items per SM it saves a split's overhead (24 to 32 pages' time) and the
+    // uneven end (about an eighth of the share).  8 decodes of up to 16,000
+    // tokens: 57.3 -> 51.9 us; 4 requests of up to 8000, 4-token spans: 57.6 -> 44.0.
+    // Below twice the least chunk the least chunk stands, whatever else is in the
+    // launch: a batch alone is then split as in a larger launch.
+    const long long share = (W + p.n_sms - 1) / p.n_sms;
+    if (share >= 2 * kMinChunkPages && share < kShortShare && (int)__reduce_add_sync(0xffffffffu, tasks) <= p.n_sms) {
+      constexpr int kTries = 12;
+      for (int i = 0; i < kTries; ++i) {
+        const int c = max(kMinChunkPages, (int)(share + (share / 8 + 32) * i / (kTries - 1)));
+        const int n = tasks ? tasks * split_count(pages, c, p.split_max) : 0;
+        if ((int)__reduce_add_sync(0xffffffffu, n) <= p.n_sms) {
+          chunk_ll = c;
+          break;
+        }
+      }
+    }
+    const int chunk = (int)min(chunk_ll, 1LL << 30);
+    int ns = 0, per = 0;
+    if (pages > 0) {
+      per = split_pages(pages, chunk, p.split_max);
+      ns = (pages + per - 1) / per;
+    }
+    int prows = ns > 1 ? ns * p.b[b].hkv * rows : 0;
+    // sort the lanes: batch by batch, the largest items first
+    uint32_t key = ((uint32_t)(IPD_MAX_BATCHES - 1 - b) << 24) |
+                   ((uint32_t)min(per, 0x7ffff) << 5) | (uint32_t)lane;
+#pragma unroll
+    for (int size = 2; size <= 32; size <<= 1) {
+#pragma unroll
+      for (int j = size >> 1; j > 0; j >>= 1) {
+        const uint32_t o = __shfl_xor_sync(0xffffffffu, key, j);
+        key = ((lane & j) == 0) == ((lane & size) == 0) ? max(key, o) : min(key, o);
+      }
+    }
+    const int src = (int)(key & 31u);
+    ns = __shfl_sync(0xffffffffu, ns, src);
+    tasks = __shfl_sync(0xffffffffu, tasks, src);
+    prows = __shfl_sync(0xffffffffu, prows, src);
+    s_pages[lane] = __shfl_sync(0xffffffffu, pages, src);
+    s_per[lane] = __shfl_sync(0xffffffffu, per, src);
+    s_rows[lane] = __shfl_sync(0xffffffffu, rows, src);
+    s_br[lane] = __shfl_sync(0xffffffffu, br, src);
+    const int item_end = warp_prefix(tasks * ns);
+    const int task_end = warp_prefix(tasks), prow_end = warp_prefix(prows);
+    s_item_end[lane] = item_end;
+    s_task0[lane] = task_end - tasks;
+    s_prow0[lane] = prow_end - prows;
+    if (lane == 31) {
+      int n = item_end;
+      if (n > p.item_cap || task_end > p.task_cap || prow_end > p.prow_cap) {
+        ipd_set_error(&g_attn_err, IPD_DEVERR_PLAN);
+        n = 0;
+      }
+      s_n_items = n;
+      p.ctrl[0] = n;
+      p.ctrl[1] = p.grid;  // the first item of every CTA is its own
+      p.ctrl[2] = task_end;
+      p.ctrl[3] = prow_end;
+      p.ctrl[4] = chunk < longest ? 1 : 0;
+    }
+  }
+  __syncthreads();
+  const int n_items = s_n_items;
+  for (int i = tid; i < n_items; i += kSmallPlanThreads) {
+    int q = 0;  // the first request whose items end past i
+#pragma unroll
+    for (int step = 16; step > 0; step >>= 1)
+      if (s_item_end[q + step - 1] <= i) q += step;
+    const int br = s_br[q], b = br >> 24, pages = s_pages[q], per = s_per[q], rows = s_rows[q];
+    const int local = i - (q > 0 ? s_item_end[q - 1] : 0);
+    const int rpb = rows_per_block(rows), nrb = (rows + rpb - 1) / rpb;
+    const int tasks = p.b[b].hkv * nrb, ns = (pages + per - 1) / per;
+    const int split = local / tasks, t = local - split * tasks;
+    const int kvh = t / nrb, rb = t - kvh * nrb;
+    const int task = s_task0[q] + t, rows_rb = min(rpb, rows - rb * rpb);
+    int4 *dst = reinterpret_cast<int4 *>(p.items + i);
+    dst[0] = make_int4(b, br & 0xffffff, kvh, rb);
+    dst[1] = make_int4(split, ns, split * per, min(pages, (split + 1) * per));
+    dst[2] = make_int4(task, ns > 1 ? s_prow0[q] + ns * (kvh * rows + rb * rpb) : -1, rows_rb,
+                       rows < kTcMinRows ? kPathCc : tc_path(rows_rb));
+    if (ns > 1 && split == 0) p.split_done[task] = 0;
   }
 }
 
@@ -1819,10 +1931,10 @@ __global__ void __launch_bounds__(kThreads, 1) attn_kernel(const __grid_constant
       const BatchDev &Bp = p.b[I.b];
       return __ldg(Bp.page_table + (long long)I.r * Bp.max_pages + pg);
     };
+    const bool late_claim = p.ctrl[4] != 0;
     int idx = blockIdx.x;  // the CTA's first item is its own
     Item I{};
     int ids = -1;
-    const bool late_claim = p.ctrl[4] != 0;
     if (idx < n_items) {
       I = p.items[idx];
       ids = load_ids(I, 0);
@@ -2268,7 +2380,9 @@ int launch(const ipd_attn_batch *const *bs, int n, float scale, void *ws, size_t
 
   // a small planner block fits beside row-pass CTAs already on an SM, so a
   // step that runs both at once does not hold the attention back
-  if (W.total_reqs <= 256 * kPlanCache)
+  if (W.total_reqs <= kSmallPlanReqs)
+    attn_plan_small_kernel<<<1, kSmallPlanThreads, 0, stream>>>(P);
+  else if (W.total_reqs <= 256 * kPlanCache)
     attn_plan_kernel<256><<<1, 256, 0, stream>>>(P);
   else
     attn_plan_kernel<kPlanThreads><<<1, kPlanThreads, 0, stream>>>(P);
