@@ -112,7 +112,9 @@ constexpr int kSizeBuckets = IPD_MAX_BATCHES * kSizesPerBatch;  // batch the lon
 static_assert(kSizeBuckets % 32 == 0, "bucket prefix: whole lanes");
 constexpr int kMaxTargetItems = 4096;            // bound used for workspace sizing
 constexpr int kMinChunkPages = 16;
-constexpr int kMergeBatch = 8;                   // splits of a merged row in flight at a time
+constexpr int kMergeBatch = 3;                   // splits of a merge's two streams in flight (with
+                                                 // four the compute region spills, long traces
+                                                 // 717 -> 724 us)
 constexpr int kSplitMax = 16;                    // splits of a task; a launch
 constexpr int kSplitMaxSmall = 32;               // of few rows may split further (its partials stay small)
 constexpr long long kSmallPartialRows = 65536;   // 32 splits of every row within this many partial rows
@@ -395,16 +397,21 @@ __device__ __forceinline__ int split_count(int pages, int chunk, int split_max) 
   return (pages + per - 1) / per;
 }
 
+// ceil(a / b), in 32 bits where a allows (a 64-bit division costs 100 ns here)
+__device__ __forceinline__ long long div_up(long long a, int b) {
+  if (a < (1LL << 31)) return ((unsigned)a + (unsigned)b - 1u) / (unsigned)b;
+  return (a + b - 1) / b;
+}
+
 // Pages per item before rounding: W pages over all tasks, the longest task
 // P_max.  Chunks of a quarter (half) of an SM's share split the long tasks for
 // balance; when no task reaches two chunks, tasks stay whole (splitting them
 // only adds item boundaries and merges: measured 3 % on 768 tasks of <= 512
 // pages over 152 SMs).
 __device__ __forceinline__ long long chunk_rule(const AttnParams &p, long long W, int P_max) {
-  const long long share = (W + p.n_sms - 1) / p.n_sms;
+  const long long share = div_up(W, p.n_sms);
   const int per_sm = share < kShortShare ? kTargetItemsShort : kTargetItemsPerSm;
-  const int target = min(kMaxTargetItems, per_sm * p.n_sms);
-  const long long chunk = (W + target - 1) / target;
+  const long long chunk = div_up(W, min(kMaxTargetItems, per_sm * p.n_sms));
   return P_max <= 2 * chunk && P_max > chunk ? P_max : chunk;
 }
 
@@ -638,6 +645,7 @@ __global__ void __launch_bounds__(kT) attn_plan_kernel(const __grid_constant__ A
 // 8-token spans: 92.2 us; in the order of the planner above 97.0, all last
 // splits at the end 102.5).
 constexpr int kSmallPlanThreads = 256;
+constexpr int kSmallPlanTries = 16;  // chunk sizes tried (two a warp)
 
 // inclusive prefix sum over the warp
 __device__ __forceinline__ int warp_prefix(int v) {
@@ -656,10 +664,12 @@ __global__ void __launch_bounds__(kSmallPlanThreads) attn_plan_small_kernel(
   // pages, pages per split, rows, and batch << 24 | request
   __shared__ int s_item_end[32], s_task0[32], s_prow0[32];
   __shared__ int s_pages[32], s_per[32], s_rows[32], s_br[32];
-  __shared__ int s_n_items;
-  const int tid = threadIdx.x, lane = tid & 31;
-  if (tid < 32) {
-    int b = 0, nrb = 0, pages = 0, rows = 0, br = 0;
+  __shared__ int s_n_items, s_share, s_longest;
+  __shared__ int s_fit[kSmallPlanTries];
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  int b = 0, nrb = 0, pages = 0, rows = 0, br = 0, tasks = 0;
+  long long chunk_ll = 0;
+  if (warp == 0) {
     if (lane < p.total_reqs) {
       b = find_batch(p, lane);
       const int r = lane - p.req_base[b];
@@ -669,30 +679,47 @@ __global__ void __launch_bounds__(kSmallPlanThreads) attn_plan_small_kernel(
       nrb = s.nrb;
       br = b << 24 | r;
     }
-    int tasks = p.b[b].hkv * nrb;
+    tasks = p.b[b].hkv * nrb;
+    s_pages[lane] = pages;
+    s_rows[lane] = tasks;
     long long W = (long long)pages * tasks;
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) W += __shfl_xor_sync(0xffffffffu, W, o);
     const int longest = __reduce_max_sync(0xffffffffu, pages);
-    long long chunk_ll = max((long long)kMinChunkPages, chunk_rule(p, W, longest));
-    // A short launch of fewer tasks than SMs: one item per SM if some chunk not
-    // much above the share cuts the tasks into no more items than that.  Against
-    // two items per SM it saves a split's overhead (24 to 32 pages' time) and the
-    // uneven end (about an eighth of the share).  8 decodes of up to 16,000
-    // tokens: 57.3 -> 51.9 us; 4 requests of up to 8000, 4-token spans: 57.6 -> 44.0.
-    // Below twice the least chunk the least chunk stands, whatever else is in the
-    // launch: a batch alone is then split as in a larger launch.
-    const long long share = (W + p.n_sms - 1) / p.n_sms;
-    if (share >= 2 * kMinChunkPages && share < kShortShare && (int)__reduce_add_sync(0xffffffffu, tasks) <= p.n_sms) {
-      constexpr int kTries = 12;
-      for (int i = 0; i < kTries; ++i) {
-        const int c = max(kMinChunkPages, (int)(share + (share / 8 + 32) * i / (kTries - 1)));
-        const int n = tasks ? tasks * split_count(pages, c, p.split_max) : 0;
-        if ((int)__reduce_add_sync(0xffffffffu, n) <= p.n_sms) {
-          chunk_ll = c;
-          break;
-        }
-      }
+    const int n_tasks = (int)__reduce_add_sync(0xffffffffu, tasks);
+    chunk_ll = max((long long)kMinChunkPages, chunk_rule(p, W, longest));
+    const long long share = div_up(W, p.n_sms);
+    if (lane == 0) {
+      s_longest = longest;
+      s_share = share >= 2 * kMinChunkPages && share < kShortShare && n_tasks <= p.n_sms ? (int)share
+                                                                                         : 0;
+    }
+  }
+  __syncthreads();
+  // A short launch of fewer tasks than SMs: one item per SM if some chunk not
+  // much above the share cuts the tasks into no more items than that.  Against
+  // two items per SM it saves a split's overhead (24 to 32 pages' time) and the
+  // uneven end (about an eighth of the share).  8 decodes of up to 16,000
+  // tokens: 57.3 -> 51.9 us; 4 requests of up to 8000, 4-token spans: 57.6 -> 44.0.
+  // Below twice the least chunk the least chunk stands, whatever else is in the
+  // launch: a batch alone is then split as in a larger launch.
+  const int share = s_share;
+  auto try_chunk = [&](int i) { return share + (share / 8 + 32) * i / (kSmallPlanTries - 1); };
+  if (share > 0) {
+    const int pg = s_pages[lane], tk = s_rows[lane];
+    for (int i = warp; i < kSmallPlanTries; i += kSmallPlanThreads / 32) {
+      const int n = tk ? tk * split_count(pg, try_chunk(i), p.split_max) : 0;
+      const int items = (int)__reduce_add_sync(0xffffffffu, n);
+      if (lane == 0) s_fit[i] = items <= p.n_sms;
+    }
+    __syncthreads();
+  }
+  if (warp == 0) {
+    const int longest = s_longest;
+    if (share > 0) {
+      const unsigned fit =
+          __ballot_sync(0xffffffffu, lane < kSmallPlanTries && s_fit[min(lane, kSmallPlanTries - 1)]);
+      if (fit) chunk_ll = try_chunk(__ffs(fit) - 1);
     }
     const int chunk = (int)min(chunk_ll, 1LL << 30);
     int ns = 0, per = 0;
@@ -762,50 +789,96 @@ __global__ void __launch_bounds__(kSmallPlanThreads) attn_plan_small_kernel(
   }
 }
 
-// Split-KV merge of one output row of a task split over several items: the
-// splits' partial rows (unnormalised O, maximum m, sum l, all in log2 units)
-// combine into the output row; lane = 4 dims, every split's loads in flight
-// at once.
-__device__ void merge_split_row(const AttnParams &p, const Item &I, int r, int lane) {
+// Split-KV merge of a task split over several items, by the CTA that finished
+// the last of them: the splits' partial rows (unnormalised O, maximum m, sum l,
+// all in log2 units) combine into the output rows.  Warp w takes rows w, w + 8,
+// ..., lane = 4 dims.  The merge ends the launch when the task was among the last
+// (64 rows of 12 splits took 18 us a row at a time), and it waits on L2: so the
+// rows' weights come first, several rows' m and l in flight (they go to `wt`,
+// [row][32] floats of the P region, which the finished item has left), then the
+// rows, in two streams of loads.  4 requests of up to 8000 tokens, 4-token spans:
+// 43.0 -> 40.5 us; a lone decode of 4096 tokens, 2 rows a task, 16.4 -> 17.9.
+__device__ void merge_split(const AttnParams &p, const Item &I, float *wt, int warp, int lane) {
   const BatchDev &Bt = p.b[I.b];
   const int q0 = Bt.cu_q[I.r], G = Bt.group;
   const int rpb = I.path != kPathCc ? kTcRows : kCcRows;
-  const int ns = I.n_split;
-  const size_t sstr = (size_t)I.rows * kPStride;
-  const float *base = p.partials + (size_t)(I.pbase + r) * kPStride;
-  const float mv = lane < ns ? __ldcg(base + lane * sstr + 128) : -INFINITY;
-  const float lv = lane < ns ? __ldcg(base + lane * sstr + 129) : 0.f;
-  const float Mx = warp_max(mv);
-  const float f = mv == -INFINITY ? 0.f : ex2_approx(mv - Mx);
-  const float Ls = warp_sum(lv * f);
-  float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+  const int ns = I.n_split, rows = I.rows;
+  const size_t sstr = (size_t)rows * kPStride;
+  const float *base = p.partials + (size_t)I.pbase * kPStride;
 #pragma unroll 1
-  for (int s0 = 0; s0 < ns; s0 += kMergeBatch) {
-    float4 ov[kMergeBatch];
+  for (int r0 = warp; r0 < rows; r0 += 4 * kCW) {
+    float mv[4], lv[4];
 #pragma unroll
-    for (int sp = 0; sp < kMergeBatch; ++sp)
-      if (s0 + sp < ns)
-        ov[sp] = __ldcg(reinterpret_cast<const float4 *>(base + (s0 + sp) * sstr) + lane);
+    for (int j = 0; j < 4; ++j) {
+      const int r = r0 + j * kCW;
+      const float *src = base + lane * sstr + (size_t)r * kPStride + 128;
+      const bool ok = r < rows && lane < ns;
+      mv[j] = ok ? __ldcg(src) : -INFINITY;
+      lv[j] = ok ? __ldcg(src + 1) : 0.f;
+    }
 #pragma unroll
-    for (int sp = 0; sp < kMergeBatch; ++sp) {
-      if (s0 + sp < ns) {
-        const float fs = __shfl_sync(0xffffffffu, f, s0 + sp);
-        acc.x = fmaf(ov[sp].x, fs, acc.x);
-        acc.y = fmaf(ov[sp].y, fs, acc.y);
-        acc.z = fmaf(ov[sp].z, fs, acc.z);
-        acc.w = fmaf(ov[sp].w, fs, acc.w);
-      }
+    for (int j = 0; j < 4; ++j) {
+      const int r = r0 + j * kCW;
+      const float Mx = warp_max(mv[j]);
+      const float f = mv[j] == -INFINITY ? 0.f : ex2_approx(mv[j] - Mx);
+      const float Ls = warp_sum(lv[j] * f);
+      if (r < rows) wt[r * 32 + lane] = Ls > 0.f ? f * (1.f / Ls) : 0.f;
     }
   }
-  const float inv = Ls > 0.f ? 1.f / Ls : 0.f;
-  const int grow = I.rb * rpb + r;
-  const int qi = grow / G, j = grow % G;
-  uint2 pk;
-  pk.x = pack_bf16x2(acc.x * inv, acc.y * inv);
-  pk.y = pack_bf16x2(acc.z * inv, acc.w * inv);
-  *reinterpret_cast<uint2 *>(Bt.out + ((size_t)(q0 + qi) * Bt.hq + I.kvh * G + j) * kD +
-                             lane * 4) = pk;
+  __syncwarp();  // (a warp reads back its own rows' weights)
+  // two streams of loads: two rows, or for at most a row a warp the row's splits
+  // k and k + kMergeBatch
+  const bool two = rows > kCW;
+  const int step = two ? kMergeBatch : 2 * kMergeBatch;
+  const size_t sv = sstr / 4;  // a split's rows, in 16-byte vectors
+#pragma unroll 1
+  for (int ra = warp; ra < rows; ra += two ? 2 * kCW : kCW) {
+    const int rb = two && ra + kCW < rows ? ra + kCW : ra;
+    const int kb = two ? 0 : kMergeBatch;
+    const float4 *pa = reinterpret_cast<const float4 *>(base + (size_t)ra * kPStride) + lane;
+    const float4 *pb = reinterpret_cast<const float4 *>(base + (size_t)rb * kPStride) + lane + kb * sv;
+    float4 A = make_float4(0.f, 0.f, 0.f, 0.f), B = A;
+#pragma unroll 1
+    for (int s0 = 0; s0 < ns; s0 += step) {
+      float4 va[kMergeBatch], vb[kMergeBatch];
+#pragma unroll
+      for (int k = 0; k < kMergeBatch; ++k) {
+        if (s0 + k < ns) va[k] = __ldcg(pa + (s0 + k) * sv);
+        if (s0 + k + kb < ns) vb[k] = __ldcg(pb + (s0 + k) * sv);
+      }
+#pragma unroll
+      for (int k = 0; k < kMergeBatch; ++k) {
+        if (s0 + k < ns) {
+          const float fa = wt[ra * 32 + s0 + k];
+          A.x = fmaf(va[k].x, fa, A.x);
+          A.y = fmaf(va[k].y, fa, A.y);
+          A.z = fmaf(va[k].z, fa, A.z);
+          A.w = fmaf(va[k].w, fa, A.w);
+        }
+        if (s0 + k + kb < ns) {
+          const float fb = wt[rb * 32 + s0 + k + kb];
+          B.x = fmaf(vb[k].x, fb, B.x);
+          B.y = fmaf(vb[k].y, fb, B.y);
+          B.z = fmaf(vb[k].z, fb, B.z);
+          B.w = fmaf(vb[k].w, fb, B.w);
+        }
+      }
+    }
+    if (!two) A = make_float4(A.x + B.x, A.y + B.y, A.z + B.z, A.w + B.w);
+    auto put = [&](int r, const float4 &v) {
+      const int grow = I.rb * rpb + r;
+      const int qi = grow / G, j = grow % G;
+      uint2 pk;
+      pk.x = pack_bf16x2(v.x, v.y);
+      pk.y = pack_bf16x2(v.z, v.w);
+      *reinterpret_cast<uint2 *>(Bt.out + ((size_t)(q0 + qi) * Bt.hq + I.kvh * G + j) * kD +
+                                 lane * 4) = pk;
+    };
+    put(ra, A);
+    if (rb != ra) put(rb, B);
+  }
 }
+static_assert(kPStride % 4 == 0, "partial rows as 16-byte vectors");
 
 // --------------------------------------------------------------------------
 // the attention kernel
@@ -843,6 +916,7 @@ struct Smem {
 };
 static_assert(Smem::off_ps + kCcW * 8 * 16 * 4 <= Smem::off_x, "CUDA-core scratch overflow");
 static_assert(kTcRows / 2 * kD * 4 <= 2 * Smem::kPHalf, "O exchange overflow");
+static_assert(kTcRows * 32 * 4 <= 2 * Smem::kPHalf, "merge weights overflow");
 static_assert(Smem::off_p % 1024 == 0, "swizzle atoms of the P tile");
 static_assert(Smem::off_bar % 8 == 0, "mbarrier alignment");
 static_assert(Smem::total <= 227 * 1024, "shared memory");
@@ -1879,7 +1953,6 @@ __global__ void __launch_bounds__(kThreads, 1) attn_kernel(const __grid_constant
   tc_fence_after();
   const uint32_t tmem = misc[0];
   dependency_wait();  // the planner's work list
-  const int n_items = p.ctrl[0];
 
   if (warp >= kCW) {
   // the third warpgroup: producer, MMA issuer, and two warps that only take
@@ -1931,14 +2004,14 @@ __global__ void __launch_bounds__(kThreads, 1) attn_kernel(const __grid_constant
       const BatchDev &Bp = p.b[I.b];
       return __ldg(Bp.page_table + (long long)I.r * Bp.max_pages + pg);
     };
+    // the CTA's first item is its own: loaded beside the counters (the list has
+    // at least a slot per CTA), looked at only if there is one
+    int idx = blockIdx.x;
+    const int n_items = p.ctrl[0];
     const bool late_claim = p.ctrl[4] != 0;
-    int idx = blockIdx.x;  // the CTA's first item is its own
-    Item I{};
+    Item I = p.items[idx];
     int ids = -1;
-    if (idx < n_items) {
-      I = p.items[idx];
-      ids = load_ids(I, 0);
-    }
+    if (idx < n_items) ids = load_ids(I, 0);
     while (idx < n_items) {
       int nxt = n_items;
       Item In = I;
@@ -2247,7 +2320,7 @@ __global__ void __launch_bounds__(kThreads, 1) attn_kernel(const __grid_constant
       named_bar_sync(1, kCW * 32);
       if (*(volatile uint32_t *)&misc[2]) {
         __threadfence();
-        for (int r = warp; r < I.rows; r += kCW) merge_split_row(p, I, r, lane);
+        merge_split(p, I, reinterpret_cast<float *>(smem + Smem::off_p), warp, lane);
       }
       named_bar_sync(1, kCW * 32);  // misc[2] is read before the next split item rewrites it
     }
