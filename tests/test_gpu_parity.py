@@ -60,6 +60,8 @@ SMALL = [
     ("one-wave-of-items", S.small_spec(n_req=9, ctx=(100, 4000), span=(1, 9)), 22),
     ("64-sub-requests", S.small_spec(n_req=32, ctx=(1, 400), span=(1, 2), vocab=512), 23),
     ("66-sub-requests", S.small_spec(n_req=33, ctx=(1, 400), span=(0, 2), vocab=512), 24),
+    # more requests: equal chunks and the rest, of any size, as the last split
+    ("chunks-and-rests", S.small_spec(n_req=36, ctx=(1, 6000), span=(1, 3), vocab=512), 25),
 ]
 
 
