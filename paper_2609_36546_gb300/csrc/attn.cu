@@ -111,6 +111,7 @@ constexpr int kSizesPerBatch = 32;                // claim order: batch by batch
 constexpr int kSizeBuckets = IPD_MAX_BATCHES * kSizesPerBatch;  // batch the longest items first
 static_assert(kSizeBuckets % 32 == 0, "bucket prefix: whole lanes");
 constexpr int kMaxTargetItems = 4096;            // bound used for workspace sizing
+constexpr int kWholePerSm = 4;                   // tasks per SM from which whole tasks even out
 constexpr int kMinChunkPages = 16;
 constexpr int kMergeBatch = 3;                   // splits of a merge's two streams in flight (with
                                                  // four the compute region spills, long traces
@@ -334,11 +335,11 @@ __device__ ReqShape req_shape(const AttnParams &p, int b, int r) {
   return s;
 }
 
-// What the first pass over the requests finds: pages over all tasks, and the
-// longest request's pages.
+// What the first pass over the requests finds: pages over all tasks, the longest
+// request's pages, and the tasks.
 struct PlanTotals {
   long long pages;
-  int longest;
+  int longest, tasks;
 };
 
 __device__ PlanTotals block_totals(PlanTotals v, PlanTotals *red) {
@@ -347,13 +348,15 @@ __device__ PlanTotals block_totals(PlanTotals v, PlanTotals *red) {
   for (int o = 16; o > 0; o >>= 1) {
     v.pages += __shfl_xor_sync(0xffffffffu, v.pages, o);
     v.longest = max(v.longest, __shfl_xor_sync(0xffffffffu, v.longest, o));
+    v.tasks += __shfl_xor_sync(0xffffffffu, v.tasks, o);
   }
   if (lane == 0) red[w] = v;
   __syncthreads();
-  PlanTotals t{0, 0};
+  PlanTotals t{0, 0, 0};
   for (int i = 0; i < nw; ++i) {
     t.pages += red[i].pages;
     t.longest = max(t.longest, red[i].longest);
+    t.tasks += red[i].tasks;
   }
   return t;
 }
@@ -418,14 +421,20 @@ __device__ __forceinline__ long long div_up(long long a, int b) {
 
 // Pages per item before rounding: W pages over all tasks, the longest task
 // P_max.  Chunks of a quarter (half) of an SM's share split the long tasks for
-// balance; when no task reaches two chunks, tasks stay whole (splitting them
-// only adds item boundaries and merges: measured 3 % on 768 tasks of <= 512
-// pages over 152 SMs).
-__device__ __forceinline__ long long chunk_rule(const AttnParams &p, long long W, int P_max) {
+// balance; when no task reaches two chunks and there are several per SM, tasks
+// stay whole: splitting them only adds item boundaries and merges (768 tasks of
+// up to 512 pages, five per SM: 352 us, split 356; 4.4 per SM 255, split 265).
+// With fewer per SM, whole tasks leave the end uneven (3.5 per SM, 33 requests of
+// up to 32,768 tokens: 1234 us, split 1169; 2.5 per SM, 32 of up to 16,000: 475
+// and 432; 1.3 per SM, 32 decodes of up to 8000: 173 and 144; 4.1 per SM: 253
+// and 245, 1.9 per SM of up to 4000 tokens: 93 and 96).
+__device__ __forceinline__ long long chunk_rule(const AttnParams &p, long long W, int P_max,
+                                                int tasks) {
   const long long share = div_up(W, p.n_sms);
   const int per_sm = share < kShortShare ? kTargetItemsShort : kTargetItemsPerSm;
   const long long chunk = div_up(W, min(kMaxTargetItems, per_sm * p.n_sms));
-  return P_max <= 2 * chunk && P_max > chunk ? P_max : chunk;
+  const bool whole = P_max <= 2 * chunk && P_max > chunk && tasks >= kWholePerSm * p.n_sms;
+  return whole ? P_max : chunk;
 }
 
 // Claim-order bucket of an item of batch `b` with `n` pages; higher buckets
@@ -510,20 +519,22 @@ __global__ void __launch_bounds__(kT) attn_plan_kernel(const __grid_constant__ A
   };
   const int n_rounds = (p.total_reqs + kT - 1) / kT;
 
-  PlanTotals mine{0, 0};
+  PlanTotals mine{0, 0, 0};
   for (int k = 0; k < n_rounds; ++k) {
     const int gi = tid + k * kT;
     if (gi < p.total_reqs) {
       int b;
       const ReqShape s = shape_of(k, gi, b);
-      mine.pages += (long long)s.pages * p.b[b].hkv * s.nrb;
+      const int tasks = s.pages > 0 ? p.b[b].hkv * s.nrb : 0;
+      mine.pages += (long long)s.pages * tasks;
+      mine.tasks += tasks;
       mine.longest = max(mine.longest, s.pages);
     }
   }
   const PlanTotals all = block_totals(mine, red);
   const long long W = all.pages;
   const int P_max = all.longest;
-  long long chunk_ll = chunk_rule(p, W, P_max);
+  long long chunk_ll = chunk_rule(p, W, P_max, all.tasks);
   if (chunk_ll < kMinChunkPages) chunk_ll = kMinChunkPages;
   if (chunk_ll > (1LL << 30)) chunk_ll = 1LL << 30;
   const int chunk = (int)chunk_ll;
@@ -701,7 +712,7 @@ __global__ void __launch_bounds__(kSmallPlanThreads) attn_plan_small_kernel(
     for (int o = 16; o > 0; o >>= 1) W += __shfl_xor_sync(0xffffffffu, W, o);
     const int longest = __reduce_max_sync(0xffffffffu, pages);
     const int n_tasks = (int)__reduce_add_sync(0xffffffffu, tasks);
-    chunk_ll = max((long long)kMinChunkPages, chunk_rule(p, W, longest));
+    chunk_ll = max((long long)kMinChunkPages, chunk_rule(p, W, longest, n_tasks));
     const long long share = div_up(W, p.n_sms);
     if (lane == 0) {
       s_longest = longest;

@@ -62,6 +62,10 @@ SMALL = [
     ("66-sub-requests", S.small_spec(n_req=33, ctx=(1, 400), span=(0, 2), vocab=512), 24),
     # more requests: equal chunks and the rest, of any size, as the last split
     ("chunks-and-rests", S.small_spec(n_req=36, ctx=(1, 6000), span=(1, 3), vocab=512), 25),
+    # tasks of one to two chunks, fewer than four per SM: split in two (12 tasks a
+    # request; the planner of at most 32 sub-requests, and the other)
+    ("halved-32-sub-requests", S.small_spec(n_req=16, ctx=(1000, 1300), span=(1, 3), vocab=512), 26),
+    ("halved-40-sub-requests", S.small_spec(n_req=20, ctx=(1000, 1300), span=(1, 3), vocab=512), 27),
 ]
 
 
