@@ -804,7 +804,7 @@ def run_next_rows(args):
                 t_draw, rows_bytes + R * V * 2, None,
                 "score pass, then one row per request re-read for the draw"),
             "sample (one row per request)": dict(row(
-                t_samp, n_dec * V * 2, o_samp, "ALU-bound: Philox + two lg2 per entry"),
+                t_samp, n_dec * V * 2, o_samp, "integer-bound: Philox of every entry, scores of the few a bound leaves"),
                 rows=n_dec, us_per_row=t_samp * 1e3 / max(n_dec, 1),
                 oracle_ms_per_row=o_samp),
             "kv_append (all span and decode rows of the step)": dict(row(
