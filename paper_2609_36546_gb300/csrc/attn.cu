@@ -110,6 +110,7 @@ constexpr int kShortShare = 800;  // pages
 constexpr int kSizesPerBatch = 32;                // claim order: batch by batch, and within a
 constexpr int kSizeBuckets = IPD_MAX_BATCHES * kSizesPerBatch;  // batch the longest items first
 static_assert(kSizeBuckets % 32 == 0, "bucket prefix: whole lanes");
+constexpr int kClaimAhead = 4;                    // stages before an item's end at which the next is claimed
 constexpr int kMaxTargetItems = 4096;            // bound used for workspace sizing
 constexpr int kWholePerSm = 4;                   // tasks per SM from which whole tasks even out
 constexpr int kMinChunkPages = 16;
@@ -179,8 +180,7 @@ struct AttnParams {
   int n_batches;
   int total_reqs;
   float scale_log2;
-  int *ctrl;       // [0] n_items, [1] dynamic item counter, [2] n_tasks, [3] partial rows,
-                   // [4] 1 if some task is split (claim the next item late)
+  int *ctrl;       // [0] n_items, [1] dynamic item counter, [2] n_tasks, [3] partial rows
   int4 *reqinfo;   // per flattened request: task offset, partial offset, n_split, (unused)
   Item *items;
   int *split_done; // per task: split items finished (the planner zeroes those of split tasks)
@@ -422,12 +422,13 @@ __device__ __forceinline__ long long div_up(long long a, int b) {
 // Pages per item before rounding: W pages over all tasks, the longest task
 // P_max.  Chunks of a quarter (half) of an SM's share split the long tasks for
 // balance; when no task reaches two chunks and there are several per SM, tasks
-// stay whole: splitting them only adds item boundaries and merges (768 tasks of
-// up to 512 pages, five per SM: 352 us, split 356; 4.4 per SM 255, split 265).
-// With fewer per SM, whole tasks leave the end uneven (3.5 per SM, 33 requests of
-// up to 32,768 tokens: 1234 us, split 1169; 2.5 per SM, 32 of up to 16,000: 475
-// and 432; 1.3 per SM, 32 decodes of up to 8000: 173 and 144; 4.1 per SM: 253
-// and 245, 1.9 per SM of up to 4000 tokens: 93 and 96).
+// stay whole: splitting them only adds item boundaries and merges (us a launch,
+// whole / split: 5.1 tasks per SM, 64 requests of up to 8192 tokens with the
+// vocabulary pass, 339 / 353; 4.7, 60 of up to 16,000, 456 / 466; 4.1, 52 of up to
+// 8192, 233 / 243).  With fewer per SM, whole tasks leave the end uneven (3.5, 33
+// of up to 32,768, 1193 / 1169; 2.5, 32 of up to 16,000, 444 / 432; 1.3, 32
+// decodes of up to 8000, 170 / 145; but 1.9, 24 of up to 4000, 89 / 96).  Tasks of
+// up to four chunks whole: 100 of up to 32,768, 7.9 per SM, 685 / 596.
 __device__ __forceinline__ long long chunk_rule(const AttnParams &p, long long W, int P_max,
                                                 int tasks) {
   const long long share = div_up(W, p.n_sms);
@@ -609,7 +610,6 @@ __global__ void __launch_bounds__(kT) attn_plan_kernel(const __grid_constant__ A
     p.ctrl[1] = p.grid;  // the first item of every CTA is its own
     p.ctrl[2] = carry.y;
     p.ctrl[3] = carry.z;
-    p.ctrl[4] = chunk < P_max ? 1 : 0;
   }
   __syncthreads();
   if (s_fail) return;
@@ -689,7 +689,7 @@ __global__ void __launch_bounds__(kSmallPlanThreads) attn_plan_small_kernel(
   // pages, pages per split, rows, and batch << 24 | request
   __shared__ int s_item_end[32], s_task0[32], s_prow0[32];
   __shared__ int s_pages[32], s_per[32], s_rows[32], s_br[32];
-  __shared__ int s_n_items, s_share, s_longest;
+  __shared__ int s_n_items, s_share;
   __shared__ int s_fit[kSmallPlanTries];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   int b = 0, nrb = 0, pages = 0, rows = 0, br = 0, tasks = 0;
@@ -715,7 +715,6 @@ __global__ void __launch_bounds__(kSmallPlanThreads) attn_plan_small_kernel(
     chunk_ll = max((long long)kMinChunkPages, chunk_rule(p, W, longest, n_tasks));
     const long long share = div_up(W, p.n_sms);
     if (lane == 0) {
-      s_longest = longest;
       s_share = share >= 2 * kMinChunkPages && share < kShortShare && n_tasks <= p.n_sms ? (int)share
                                                                                          : 0;
     }
@@ -740,7 +739,6 @@ __global__ void __launch_bounds__(kSmallPlanThreads) attn_plan_small_kernel(
     __syncthreads();
   }
   if (warp == 0) {
-    const int longest = s_longest;
     if (share > 0) {
       const unsigned fit =
           __ballot_sync(0xffffffffu, lane < kSmallPlanTries && s_fit[min(lane, kSmallPlanTries - 1)]);
@@ -789,7 +787,6 @@ __global__ void __launch_bounds__(kSmallPlanThreads) attn_plan_small_kernel(
       p.ctrl[1] = p.grid;  // the first item of every CTA is its own
       p.ctrl[2] = task_end;
       p.ctrl[3] = prow_end;
-      p.ctrl[4] = chunk < longest ? 1 : 0;
     }
   }
   __syncthreads();
@@ -1989,11 +1986,13 @@ __global__ void __launch_bounds__(kThreads, 1) attn_kernel(const __grid_constant
     // Page ids are read 32 at a time (one coalesced load per warp), one batch
     // ahead of use, and the next item's descriptor is fetched while the
     // current one streams, so no TMA issue waits on a global load.
-    // When the planner split tasks into chunks of about equal size, the next
-    // item is claimed four stages before the current one ends, so that the
-    // CTA that frees up first takes it (2 % off a launch whose tasks split).
-    // With whole tasks of very different sizes, claiming it as the current
-    // one starts measured as good or better.
+    // The next item is claimed four stages before the current one ends, so that
+    // the CTA that frees up first takes it and none sits on an item it cannot
+    // start.  Claimed as an item starts, us a launch, against four stages before
+    // its end: 64 requests of up to 8192 tokens with the vocabulary pass 352 / 342,
+    // 52 of up to 8192 253 / 235, 33 of up to 32,768 1207 / 1168; nothing lost.
+    // Two, three or six stages are within 0.5 % (six: 32 decodes of up to 4000
+    // tokens 61.6 -> 64.3).
     const uint64_t policy = l2_policy_evict_first();
     uint32_t it = 0;
     bool aborted = false;
@@ -2034,7 +2033,6 @@ __global__ void __launch_bounds__(kThreads, 1) attn_kernel(const __grid_constant
     // at least a slot per CTA), looked at only if there is one
     int idx = blockIdx.x;
     const int n_items = p.ctrl[0];
-    const bool late_claim = p.ctrl[4] != 0;
     Item I = p.items[idx];
     int ids = -1;
     if (idx < n_items) ids = load_ids(I, 0);
@@ -2048,7 +2046,7 @@ __global__ void __launch_bounds__(kThreads, 1) attn_kernel(const __grid_constant
       const int nst = (npages + kStagePages - 1) / kStagePages;
       int ids_next = (npages > 32) ? load_ids(I, 1) : -1;
       int ids_item_next = -1;
-      const int st_claim = late_claim ? max(0, nst - 4) : 0;
+      const int st_claim = max(0, nst - kClaimAhead);
       const int st_take = min(nst - 1, st_claim + 1);
       for (int st = 0; st < nst; ++st) {
         if (st == st_claim) claim_issue();
