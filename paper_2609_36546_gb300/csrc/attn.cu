@@ -190,8 +190,21 @@ struct AttnParams {
   long long prow_cap;
   int split_max;     // most splits of a task (at most 32: one partial per lane of a merging warp)
   int n_sms;
-  int grid;          // CTAs of the attention kernel; CTA i starts with item i
+  int grid;          // CTAs of the attention kernel
+  int first_half;    // CTA i starts with item i, or (> 0) as first_item() says
 };
+
+// The item that CTA `cta` starts with.  Where tasks have several row blocks, their
+// items follow one another in the list, and items 2 i and 2 i + 1 go to CTAs i and
+// i + grid / 2: the two read the same K and V, and streamed from neighbouring CTAs
+// they were slower (us a launch, CTA i with item i / this: 33 requests of up to
+// 32,768 tokens with 24-token spans 1169 / 1028, 64 of up to 8192 with 20 385 /
+// 363, 24 of up to 8192 with 24 228 / 188).  Where no task has two, CTA i keeps
+// item i (8 decodes of up to 16,000 tokens 50.0, spread 50.2, claimed 51.5).
+__device__ __forceinline__ int first_item(int cta, int half) {
+  if (cta >= 2 * half) return cta;
+  return cta < half ? 2 * cta : 2 * (cta - half) + 1;
+}
 
 struct StageMeta {
   int item;
@@ -2029,9 +2042,9 @@ __global__ void __launch_bounds__(kThreads, 1) attn_kernel(const __grid_constant
       const BatchDev &Bp = p.b[I.b];
       return __ldg(Bp.page_table + (long long)I.r * Bp.max_pages + pg);
     };
-    // the CTA's first item is its own: loaded beside the counters (the list has
+    // the CTA's first item is its own (first_item): loaded beside the counters (the list has
     // at least a slot per CTA), looked at only if there is one
-    int idx = blockIdx.x;
+    int idx = first_item(blockIdx.x, p.first_half);
     const int n_items = p.ctrl[0];
     Item I = p.items[idx];
     int ids = -1;
@@ -2474,6 +2487,8 @@ int launch(const ipd_attn_batch *const *bs, int n, float scale, void *ws, size_t
   P.split_max = W.split_max;
   P.n_sms = D.sms;
   P.grid = std::max(1, std::min(D.sms, W.item_cap));
+  for (int i = 0; i < n; ++i)
+    if ((long long)P.b[i].max_q_len * P.b[i].group > kTcRows) P.first_half = P.grid / 2;
 
   // a small planner block fits beside row-pass CTAs already on an SM, so a
   // step that runs both at once does not hold the attention back

@@ -66,6 +66,9 @@ SMALL = [
     # request; the planner of at most 32 sub-requests, and the other)
     ("halved-32-sub-requests", S.small_spec(n_req=16, ctx=(1000, 1300), span=(1, 3), vocab=512), 26),
     ("halved-40-sub-requests", S.small_spec(n_req=20, ctx=(1000, 1300), span=(1, 3), vocab=512), 27),
+    # two row blocks a task, more items than CTAs: a task's two start on different halves
+    ("pairs-of-row-blocks", S.small_spec(n_req=20, ctx=(100, 900), span=(17, 20), direction="S",
+                                         vocab=512), 28),
 ]
 
 
